@@ -122,14 +122,14 @@ template <typename T>
 static int32_t run_steps(const std::vector<Step>& plan, int i0, int i1, const int32_t* rowptr,
                          const int32_t* colind, const T* vals, int32_t n, int64_t nnz,
                          const Buffers& bufs, cudaStream_t s, double* bytes_out,
-                         bool reserve_l2 = true);
+                         bool reserve_l2 = true, DiagStore* diag = nullptr);
 
 template <typename T>
 int32_t run_plan(const std::vector<Step>& plan, const int32_t* rowptr, const int32_t* colind,
                  const T* vals, int32_t n, int64_t nnz, const Buffers& bufs, cudaStream_t s,
-                 double* bytes_out, bool reserve_l2) {
+                 double* bytes_out, bool reserve_l2, DiagStore* diag) {
     return run_steps<T>(plan, 0, (int)plan.size(), rowptr, colind, vals, n, nnz, bufs, s,
-                        bytes_out, reserve_l2);
+                        bytes_out, reserve_l2, diag);
 }
 
 // steps [i0, i1) of a plan, in order
@@ -137,7 +137,7 @@ template <typename T>
 static int32_t run_steps(const std::vector<Step>& plan, int i0, int i1, const int32_t* rowptr,
                          const int32_t* colind, const T* vals, int32_t n, int64_t nnz,
                          const Buffers& bufs, cudaStream_t s, double* bytes_out,
-                         bool reserve_l2) {
+                         bool reserve_l2, DiagStore* diag) {
     double bytes = 0.0;
     int32_t keep_rows = 0;
     const int keep = keep_a_flag(n, nnz, (int)sizeof(T), 3, reserve_l2, &keep_rows);
@@ -167,6 +167,7 @@ static int32_t run_steps(const std::vector<Step>& plan, int i0, int i1, const in
         a.flags = st.flags | keep;
         a.keep_rows = keep_rows;
         a.part = nullptr;
+        if (diag) diag->give(a);
         int32_t rc = launch_step<T>(st.op, a, s);
         if (rc < 0) return rc;
         bytes += step_bytes(st.op, st.flags, n, nnz, (int)sizeof(T));
@@ -177,10 +178,10 @@ static int32_t run_steps(const std::vector<Step>& plan, int i0, int i1, const in
 
 template int32_t run_plan<double>(const std::vector<Step>&, const int32_t*, const int32_t*,
                                   const double*, int32_t, int64_t, const Buffers&, cudaStream_t,
-                                  double*, bool);
+                                  double*, bool, DiagStore*);
 template int32_t run_plan<float>(const std::vector<Step>&, const int32_t*, const int32_t*,
                                  const float*, int32_t, int64_t, const Buffers&, cudaStream_t,
-                                 double*, bool);
+                                 double*, bool, DiagStore*);
 
 // ---------------------------------------------------------------------------
 // Workspace: one stream-ordered allocation carved into aligned pieces
@@ -318,6 +319,7 @@ struct SolveCore {
     OrthoWs ows{};
     GmresState gs{};
     std::vector<Step> phi_plan, p_plan;
+    DiagStore diag;   // flexible form: A32 by diagonals
     ppg_stats st{};
 };
 
@@ -559,6 +561,9 @@ static int32_t run_solve(SolveCore& c) {
     if (!std::isfinite(beta)) return PPG_ERR_NONFINITE;
     bool converged = c.st.true_relres <= c.tol;
 
+    if (pp && c.flex && !c.sweep && !converged)
+        PPG_TRY(c.diag.build(c.A32->rowptr, c.A32->colind, (const float*)c.A32->vals, n, nnz,
+                             4 * (int64_t)c.p_plan.size(), s));   // (several outer steps)
     Buffers phib{};
     phib.ptr[B_A] = c.va;
     phib.ptr[B_B] = c.vb;
@@ -603,7 +608,7 @@ static int32_t run_solve(SolveCore& c) {
             fb.ptr[B_B] = c.fb;
             fb.ptr[B_C] = c.fc;
             return run_steps<float>(c.p_plan, i0, i1, c.A32->rowptr, c.A32->colind,
-                                    (const float*)c.A32->vals, n, nnz, fb, s, by);
+                                    (const float*)c.A32->vals, n, nnz, fb, s, by, true, &c.diag);
         }
         phib.ptr[B_IN] = c.V + (size_t)j * c.ldv;
         phib.ptr[B_OUT] = c.V + (size_t)(j + 1) * c.ldv;
@@ -1146,9 +1151,14 @@ static int32_t apply_common(const ppg_csr* A, const ppg_roots* r, const void* v,
     if (A->dtype == PPG_F64)
         rc = run_plan<double>(plan, A->rowptr, A->colind, (const double*)A->vals, A->n, A->nnz,
                               bufs, s, nullptr);
-    else
-        rc = run_plan<float>(plan, A->rowptr, A->colind, (const float*)A->vals, A->n, A->nnz,
-                             bufs, s, nullptr);
+    else {
+        DiagStore diag;
+        rc = diag.build(A->rowptr, A->colind, (const float*)A->vals, A->n, A->nnz,
+                        (int64_t)plan.size(), s);
+        if (rc == PPG_OK)
+            rc = run_plan<float>(plan, A->rowptr, A->colind, (const float*)A->vals, A->n, A->nnz,
+                                 bufs, s, nullptr, true, &diag);
+    }
     ar.release(s);
     return rc;
 }

@@ -127,6 +127,24 @@ enum StepFlag : int {
     F_PZERO = 2,   // P_*: the accumulator p starts at zero (a1 not read)
     F_NO_O1 = 4,   // P_PAIR1: tmp not needed afterwards
     F_KEEP_A = 8,  // copy A with an L2 evict-last hint (A and the vectors fit in L2)
+    F_SERIAL = 16, // not a programmatic dependent: the first step that reads a
+                   // diagonal form built by the kernel before it
+};
+
+// An FP32 matrix by its diagonals (spmv_root.cu), built on the device inside
+// the call that uses it.  head: [0] != 0: the matrix has no such form, [1]
+// diagonals, [2] bit q: diagonal q has one value throughout, then the column -
+// row offsets in ascending order.
+constexpr int DIAG_MAX = 32;
+constexpr int DIAG_HEAD = 4 + DIAG_MAX;
+constexpr int DIAG_PAD = 512;   // rows of a diagonal are padded to whole tiles of any step
+struct DiagForm {
+    const int32_t* head;   // nullptr: none
+    const float* same;     // [DIAG_MAX] the one value of such diagonals
+    const float* vals;     // [diagonals][ld] the others, row by row
+    const void* mask;      // [ld] bit q of row r: the row has an entry on diagonal q
+    int32_t ld;
+    int32_t mask_bytes;    // 1, 2 or 4
 };
 
 template <typename T>
@@ -148,6 +166,7 @@ struct StepArgs {
     int32_t keep_rows;  // rows [0, keep_rows) stage their nonzeros with an L2
                         // evict-last hint (a chain over a matrix too large
                         // for L2 keeps its leading rows resident)
+    DiagForm diag;      // FP32: the same matrix by diagonals (diag.head != nullptr)
 };
 
 // Systems of at most DIRECT_MAX_N rows take the direct-read variant of the
@@ -181,6 +200,28 @@ int keep_a_flag(int64_t n, int64_t nnz, int elem, int nvec, bool may_reserve = t
 // at least the partial sums any residual step of n rows writes (one per CTA)
 int32_t spmv_grid_blocks(int32_t n);
 
+// The diagonal form of an FP32 matrix for `steps` root steps to come: null
+// where it does not pay or there is no memory for it.  A call's own, released
+// with it.
+struct DiagStore {
+    DiagForm f{};
+    bool fresh = false;    // no step has read it yet
+    void* mem = nullptr;
+    cudaStream_t s = nullptr;
+    int32_t build(const int32_t* rowptr, const int32_t* colind, const float* vals, int32_t n,
+                  int64_t nnz, int64_t steps, cudaStream_t stream);
+    // hand it to a step
+    template <typename T>
+    void give(StepArgs<T>& a) {
+        a.diag = f;
+        if (f.head && fresh) a.flags |= F_SERIAL;
+        fresh = false;
+    }
+    ~DiagStore() {
+        if (mem) cudaFreeAsync(mem, s);
+    }
+};
+
 // algorithmic bytes of one fused step
 double step_bytes(int op, int flags, int64_t n, int64_t nnz, int elem);
 
@@ -211,7 +252,7 @@ template <typename T>
 int32_t run_plan(const std::vector<Step>& plan, const int32_t* rowptr,
                  const int32_t* colind, const T* vals, int32_t n, int64_t nnz,
                  const Buffers& bufs, cudaStream_t s, double* bytes_out,
-                 bool reserve_l2 = true);
+                 bool reserve_l2 = true, DiagStore* diag = nullptr);
 
 // ---------------------------------------------------------------------------
 // Multi-root fused sweep (sweep.cu): Algorithm 3 on a plan's reordered FP32

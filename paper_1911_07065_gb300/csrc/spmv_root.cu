@@ -32,6 +32,7 @@
 // holds the nonzeros of its leading rows that way in a 48 MB set-aside and
 // streams the rest with evict-first, prefetching it into L2 half a resident
 // wave ahead.
+#include <algorithm>
 #include <atomic>
 
 #include "ppg_common.cuh"
@@ -152,6 +153,20 @@ __device__ __forceinline__ void step_epilogue(const StepArgs<T>& a, int64_t r, T
     }
 }
 
+// part[block] = the sum of sq over the CTA's NT threads, in a fixed order
+template <int NT>
+__device__ __forceinline__ void block_sq(double sq, double* sred, double* part) {
+    const int tid = threadIdx.x;
+    for (int off = 16; off > 0; off >>= 1) sq += __shfl_down_sync(0xffffffffu, sq, off);
+    if ((tid & 31) == 0) sred[tid >> 5] = sq;
+    __syncthreads();
+    if (tid == 0) {
+        double t = 0.0;
+        for (int w = 0; w < NT / 32; ++w) t += sred[w];
+        part[blockIdx.x] = t;
+    }
+}
+
 // Rows per thread: FP32 tiles take two rows per thread (512 rows per CTA),
 // so each CTA's latency-bound phases (row pointers, staging, gathers) serve
 // twice the bytes; FP64 keeps one (at 32 registers, 2048 threads per SM).
@@ -217,9 +232,378 @@ __device__ __forceinline__ T row_dot(const T* sval, const int32_t* scol, const T
     return acc;
 }
 
+// ---------------------------------------------------------------------------
+// Diagonal form (FP32)
+// ---------------------------------------------------------------------------
+//
+// A matrix from a grid has few distinct column - row offsets.  Stored by these
+// diagonals -- a sorted list of offsets, a bit per row and offset, the values
+// diagonal by diagonal -- a step reads no column indices and no row pointers,
+// a diagonal with one value throughout is not read at all, and all that a tile
+// of rows needs of x is a few contiguous windows, which the bulk-copy engine
+// brings to shared memory in one round trip.  Rows are still summed entry by
+// entry in stored order (the form is built only where the columns of every row
+// increase, as the offsets then do), so the results are those of the CSR steps
+// bit for bit.
+//
+// Building it is two passes over the matrix, inside the call.  Whether the
+// matrix has the form is known on the device alone: the steps read it from
+// the head and take the CSR path if not, so the host waits for nothing, and
+// the call stays asynchronous and can be captured.
+//
+// 160^3, FP32, 60 steps of p(A): 2.94 -> 1.52 ms (one value per diagonal), 2.93
+// -> 2.15 ms (values of their own), against 49 us a step at 0.91 of the copy
+// bandwidth by CSR.  What is left is the issue of instructions (two thirds of
+// the slots) and the life of a CTA (head, copies, arithmetic: three trips).
+// Tried and slower: reading x and the values straight from global memory (27 -
+// 35 us a step, five dependent trips per CTA), and CTAs that stay and loop over
+// tiles without copies in flight (26 - 37 us).
+//
+// FP64 steps have no use for it: their multiply-adds bound them (504 G FMA/s
+// measured, 1.6 per clock and SM; the chains run at 0.85 - 0.89 of that).
+
+constexpr int32_t DIAG_NONE = INT32_MAX;   // no offset: columns are below n
+
+// the head and, behind it, the finder's list
+struct DiagHead {
+    int32_t w[DIAG_HEAD];
+    int32_t off[DIAG_MAX];            // unsorted, DIAG_NONE: free
+    uint32_t ref[DIAG_MAX];           // bits of the first value seen, DIAG_UNSET: none yet
+    uint32_t mixed;                   // bit i: list entry i has several values
+};
+constexpr uint32_t DIAG_UNSET = 0x7fb4deadu;   // a NaN that no arithmetic returns
+
+__global__ void k_diag_init(DiagHead* H) {
+    const int i = threadIdx.x;
+    if (i < DIAG_HEAD) H->w[i] = 0;
+    if (i < DIAG_MAX) {
+        H->off[i] = DIAG_NONE;
+        H->ref[i] = DIAG_UNSET;
+    }
+    if (i == 0) H->mixed = 0;
+}
+
+// Every offset of the matrix into the list, and whether its values are all the
+// same.  A CTA takes DIAG_ROWS rows: each round it finds the rows' smallest
+// next offset, the rows that hold it and whether their values agree; at the
+// end one warp compares its findings with the list and adds what is new.
+constexpr int DIAG_ROWS = 128;
+__global__ void __launch_bounds__(DIAG_ROWS)
+k_diag_find(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colind,
+            const float* __restrict__ vals, int32_t n, int32_t most, DiagHead* H) {
+    constexpr int NW = DIAG_ROWS / 32;
+    __shared__ int32_t s_min[2][NW];
+    __shared__ int32_t s_off[DIAG_MAX];
+    __shared__ uint32_t s_ref[DIAG_MAX];
+    __shared__ int s_bad;
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (tid == 0) s_bad = *(volatile int32_t*)&H->w[0];
+    __syncthreads();
+    if (s_bad) return;   // another CTA has seen that there is no such form
+    const int64_t r = (int64_t)blockIdx.x * DIAG_ROWS + tid;
+    int32_t k = 0, e = 0;
+    if (r < n) {
+        k = __ldg(rowptr + r);
+        e = __ldg(rowptr + r + 1);
+    }
+    int32_t cur = k < e ? __ldg(colind + k) - (int32_t)r : DIAG_NONE;
+    bool ok = true;
+    unsigned mixed = 0;
+    int q = 0;
+    for (;; ++q) {
+        const int32_t wm = __reduce_min_sync(0xffffffffu, cur);
+        if (lane == 0) s_min[q & 1][tid >> 5] = wm;
+        __syncthreads();
+        int32_t m = s_min[q & 1][0];
+#pragma unroll
+        for (int w = 1; w < NW; ++w) m = min(m, s_min[q & 1][w]);
+        if (m == DIAG_NONE || q == most) {   // uniform
+            ok = ok && m == DIAG_NONE;
+            break;
+        }
+        const bool hit = cur == m;
+        uint32_t v = 0;
+        if (hit) {
+            v = __float_as_uint(__ldg(vals + k));
+            s_ref[q] = v;   // any of them
+            s_off[q] = m;
+            ++k;
+            cur = k < e ? __ldg(colind + k) - (int32_t)r : DIAG_NONE;
+            ok = ok && cur > m;   // columns increase within the row
+        }
+        __syncthreads();
+        if (!__syncthreads_and(!hit || v == s_ref[q])) mixed |= 1u << q;
+    }
+    ok = __syncthreads_and(ok);
+    if (!ok) {
+        if (tid == 0) atomicExch(&H->w[0], 1);
+        return;
+    }
+    if (tid >= 32) return;
+    // lane i < q: this CTA's offset i against the list (one load), then
+    // whatever the list does not have yet
+    const int32_t have = *(volatile int32_t*)&H->off[lane];
+    const unsigned gmixed = *(volatile uint32_t*)&H->mixed;
+    const int32_t mine = lane < q ? s_off[lane] : DIAG_NONE;
+    int slot = -1;
+    for (int i = 0; i < DIAG_MAX; ++i)
+        if (__shfl_sync(0xffffffffu, have, i) == mine && mine != DIAG_NONE) slot = i;
+    if (mine != DIAG_NONE && slot < 0)
+        for (int i = 0; i < DIAG_MAX && slot < 0; ++i) {
+            const int32_t old = atomicCAS(&H->off[i], DIAG_NONE, mine);
+            if (old == DIAG_NONE || old == mine) slot = i;
+        }
+    if (mine != DIAG_NONE) {
+        if (slot < 0) {
+            atomicExch(&H->w[0], 1);
+        } else if (!((gmixed >> slot) & 1)) {
+            const uint32_t v = s_ref[lane];
+            uint32_t ref = *(volatile uint32_t*)&H->ref[slot];
+            if (ref == DIAG_UNSET) {
+                ref = atomicCAS(&H->ref[slot], DIAG_UNSET, v);
+                if (ref == DIAG_UNSET) ref = v;
+            }
+            if (((mixed >> lane) & 1) || ref != v || v == DIAG_UNSET)
+                atomicOr(&H->mixed, 1u << slot);
+        }
+    }
+}
+
+// the form itself, one row per thread, from the finished list
+__global__ void __launch_bounds__(256)
+k_diag_fill(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colind,
+            const float* __restrict__ vals, int32_t n, int32_t most, DiagHead* H, float* same, float* out,
+            int32_t ld, void* mask, int32_t mask_bytes) {
+    __shared__ int32_t s_off[DIAG_MAX];
+    __shared__ unsigned s_same;
+    const int tid = threadIdx.x;
+    if (tid < 32) {
+        const int32_t o = H->off[tid];
+        const bool used = o != DIAG_NONE;
+        const int nq = __popc(__ballot_sync(0xffffffffu, used));
+        int rank = 0;
+        for (int i = 0; i < DIAG_MAX; ++i) rank += __shfl_sync(0xffffffffu, o, i) < o;
+        const bool one = used && !((H->mixed >> tid) & 1);
+        const unsigned bits = __reduce_or_sync(0xffffffffu, one ? 1u << rank : 0u);
+        const bool bad = nq > most || *(volatile int32_t*)&H->w[0] != 0;
+        if (used) s_off[rank] = o;
+        if (tid == 0) s_same = bad ? 0xffffffffu : bits;
+        if (blockIdx.x == 0) {
+            if (used) {
+                H->w[4 + rank] = o;
+                if (one) same[rank] = __int_as_float((int)H->ref[tid]);
+            }
+            if (tid == 0) {
+                H->w[1] = nq;
+                H->w[2] = (int32_t)bits;
+                if (bad) H->w[0] = 1;
+            }
+        }
+        __syncwarp();
+        if (bad && tid == 0) s_off[0] = DIAG_NONE;
+    }
+    __syncthreads();
+    if (s_off[0] == DIAG_NONE) return;
+    const unsigned same_bits = s_same;
+    const int64_t r = (int64_t)blockIdx.x * 256 + tid;
+    if (r >= n) return;
+    const int32_t e = __ldg(rowptr + r + 1);
+    unsigned bits = 0;
+    int q = 0;
+    for (int32_t k = __ldg(rowptr + r); k < e; ++k, ++q) {
+        const int32_t o = __ldg(colind + k) - (int32_t)r;
+        while (s_off[q] != o) ++q;
+        bits |= 1u << q;
+        if (!((same_bits >> q) & 1)) out[(int64_t)q * ld + r] = __ldg(vals + k);
+    }
+    if (mask_bytes == 1)
+        ((uint8_t*)mask)[r] = (uint8_t)bits;
+    else if (mask_bytes == 2)
+        ((uint16_t*)mask)[r] = (uint16_t)bits;
+    else
+        ((uint32_t*)mask)[r] = bits;
+}
+
+// where a tile's diagonals lie in its shared memory, in bytes
+constexpr int32_t DIAG_SAME = INT32_MIN;
+struct DiagSlot {
+    int32_t x;       // the first row's entry of x
+    int32_t v;       // the first row's value; DIAG_SAME: the value is `same`
+    float same;
+    int32_t off;
+};
+
+__device__ __forceinline__ unsigned diag_bits(const DiagForm& f, int32_t r) {
+    return f.mask_bytes == 1 ? __ldg((const uint8_t*)f.mask + r)
+           : f.mask_bytes == 2 ? __ldg((const uint16_t*)f.mask + r)
+                               : __ldg((const uint32_t*)f.mask + r);
+}
+
+__device__ __forceinline__ void bulk_to_shared(uint32_t dst, const void* src, uint32_t bytes,
+                                               uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+            dst),
+        "l"(src), "r"(bytes), "r"(bar)
+        : "memory");
+}
+
+constexpr uint32_t DIAG_SPIN_LIMIT = 1u << 20;   // polls of a copy's barrier (some 0.1 s)
+
+__device__ __forceinline__ bool diag_arrived(uint32_t bar) {
+    for (uint32_t it = 0; it < DIAG_SPIN_LIMIT; ++it) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(bar)
+            : "memory");
+        if (ok) return true;
+    }
+    return false;
+}
+
+// One tile of a step by diagonals: ROWS rows from row0, NT threads, thread tid
+// on rows tid + i NT.  Warp 0 merges offsets less than 16 apart into windows
+// of x, lays windows and values out in the CAP elements of `sm`, and issues
+// the copies: values before the wait on the previous step, windows after it.
+// A tile whose data does not fit (many diagonals with values of their own)
+// reads global memory instead.
+template <typename T, int OP, int NT, int RPT, int CAP>
+__device__ __forceinline__ void diag_tile(const StepArgs<T>& a, int32_t row0, int nrows, float* sm,
+                                          DiagSlot* slot, uint64_t* bar, int* info, double& sq) {
+    constexpr int ROWS = NT * RPT;
+    const DiagForm& f = a.diag;
+    const int tid = threadIdx.x;
+    const uint32_t mb = (uint32_t)__cvta_generic_to_shared(bar);
+    unsigned b[RPT];
+#pragma unroll
+    for (int i = 0; i < RPT; ++i)
+        b[i] = tid + i * NT < nrows ? diag_bits(f, row0 + tid + i * NT) : 0;
+    const int nq = __ldg(f.head + 1);
+    if (tid < 32) {
+        const int lane = tid;
+        const unsigned same = (unsigned)__ldg(f.head + 2);
+        const bool used = lane < nq;
+        const int32_t o = used ? __ldg(f.head + 4 + lane) : 0;
+        const int32_t before = __shfl_up_sync(0xffffffffu, o, 1);
+        const bool opens = used && (lane == 0 || o - before > 16);
+        const unsigned heads = __ballot_sync(0xffffffffu, opens);
+        const unsigned upto = 0xffffffffu >> (31 - lane);
+        const int first = 31 - __clz(heads & upto | 1u);
+        const unsigned later = heads & ~upto;
+        const int last = later ? __ffs(later) - 2 : nq - 1;
+        const int32_t ws = __shfl_sync(0xffffffffu, o, first);
+        const int32_t we = __shfl_sync(0xffffffffu, o, max(last, 0));
+        // the window's elements [lo, hi) of x, on 16-byte boundaries
+        const int32_t lo = max(row0 + ws, 0), hi = min(row0 + nrows + we, a.n);
+        const unsigned skew = ((unsigned)(uintptr_t)(a.x + lo) & 15u) / 4;
+        const unsigned bytes_to = ((unsigned)(hi - lo) + skew + 3) / 4 * 16;
+        // places: windows first, then the diagonals with values of their own
+        const int32_t room = opens ? (ROWS + (we - ws) + 8 + 3) / 4 * 4 : 0;
+        int32_t end = room;
+#pragma unroll
+        for (int s = 1; s < 32; s <<= 1) {
+            const int32_t v = __shfl_up_sync(0xffffffffu, end, s);
+            if (lane >= s) end += v;
+        }
+        const int32_t at = __shfl_sync(0xffffffffu, end - room, first);
+        const int32_t xs = __shfl_sync(0xffffffffu, end, 31);
+        const bool own = used && !((same >> lane) & 1);
+        const unsigned owns = __ballot_sync(0xffffffffu, own);
+        const int32_t vat = xs + __popc(owns & (upto >> 1)) * ROWS;
+        const bool fits = xs + __popc(owns) * ROWS <= CAP;
+        if (used)
+            slot[lane] = {(at + (int32_t)skew + (row0 + o - lo)) * 4, own ? vat * 4 : DIAG_SAME,
+                          own ? 0.0f : __ldg(f.same + lane), o};
+        const uint32_t bytes = opens && hi > lo ? bytes_to : 0;
+        const uint32_t total = __reduce_add_sync(0xffffffffu, bytes) + __popc(owns) * (ROWS * 4u);
+        if (lane == 0) {
+            info[0] = nq;
+            info[1] = fits;
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb) : "memory");
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb),
+                         "r"(fits ? total : 0u)
+                         : "memory");
+        }
+        __syncwarp();
+        const uint32_t base = (uint32_t)__cvta_generic_to_shared(sm);
+        if (fits && own)
+            bulk_to_shared(base + vat * 4, f.vals + (int64_t)lane * f.ld + row0, ROWS * 4, mb);
+        // the vectors written by the previous step are complete and visible
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (fits && bytes) bulk_to_shared(base + at * 4, a.x + lo - (int)skew, bytes, mb);
+    } else {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+    }
+    T e0[RPT], e1[RPT], e2[RPT], acc[RPT];
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+        e0[i] = e1[i] = e2[i] = acc[i] = T(0);
+        const int64_t r = (int64_t)row0 + tid + i * NT;
+        if (tid + i * NT < nrows) {
+            if (a.a0) e0[i] = __ldg(a.a0 + r);
+            if (a.a1 && !(a.flags & F_PZERO)) e1[i] = a.a1[r];
+            if (a.a2 && (a.flags & F_FINAL)) e2[i] = __ldg(a.a2 + r);
+        }
+    }
+    __syncthreads();
+    const bool ready = diag_arrived(mb);
+    if (ready && info[1]) {
+        // rows that lack a diagonal only where a grid ends: most warps have none
+        const unsigned all = 0xffffffffu >> (32 - nq);
+        bool whole = true;
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) whole = whole && b[i] == all;
+        const char* me = reinterpret_cast<const char*>(sm + tid);
+        auto at = [&](int32_t off, int i) {
+            return *reinterpret_cast<const float*>(me + off + i * NT * (int)sizeof(float));
+        };
+        if (__all_sync(0xffffffffu, whole)) {
+#pragma unroll 4
+            for (int q = 0; q < nq; ++q) {
+                const DiagSlot s = slot[q];
+#pragma unroll
+                for (int i = 0; i < RPT; ++i)
+                    acc[i] = fma(s.v == DIAG_SAME ? s.same : at(s.v, i), at(s.x, i), acc[i]);
+            }
+        } else {
+#pragma unroll 4
+            for (int q = 0; q < nq; ++q) {
+                const DiagSlot s = slot[q];
+#pragma unroll
+                for (int i = 0; i < RPT; ++i)
+                    if ((b[i] >> q) & 1)
+                        acc[i] = fma(s.v == DIAG_SAME ? s.same : at(s.v, i), at(s.x, i), acc[i]);
+            }
+        }
+    } else {   // no room, or the copies did not arrive: from global memory
+        for (int q = 0; q < nq; ++q) {
+            const DiagSlot s = slot[q];
+#pragma unroll
+            for (int i = 0; i < RPT; ++i)
+                if ((b[i] >> q) & 1) {
+                    const int64_t r = (int64_t)row0 + tid + i * NT;
+                    acc[i] = fma(s.v == DIAG_SAME ? s.same : __ldg(f.vals + (int64_t)q * f.ld + r),
+                                 __ldg(a.x + r + s.off), acc[i]);
+                }
+        }
+        if (!ready) diag_arrived(mb);   // nothing may land in this CTA's memory after it
+    }
+#pragma unroll
+    for (int i = 0; i < RPT; ++i)
+        if (tid + i * NT < nrows)
+            step_epilogue<T, OP>(a, (int64_t)row0 + tid + i * NT, acc[i], e0[i], e1[i], e2[i], sq);
+}
+
 // PF: prefetch the tile a.pf_ahead tiles ahead (half a resident wave) into
 // L2 (launched when the matrix is not held in an L2 set-aside)
-template <typename T, int OP, bool PF>
+// DG: the (FP32) matrix is at hand by its diagonals too, if it has that form
+template <typename T, int OP, bool PF, bool DG>
 __global__ void __launch_bounds__(step_threads<T>(), step_min_ctas<T, OP>())
 k_spmv_step(const StepArgs<T> a) {
     constexpr int NT = step_threads<T>();      // threads per CTA
@@ -228,8 +612,9 @@ k_spmv_step(const StepArgs<T> a) {
     constexpr int RPT = step_rpt<T>();
     constexpr int ROWS = NT * RPT;      // rows per CTA
     constexpr int CHUNK = step_chunk<T>();     // nonzeros staged per chunk
-    __shared__ __align__(16) T sval[CHUNK + PAD];
-    __shared__ __align__(16) int32_t scol[CHUNK + PAD];
+    __shared__ __align__(16) unsigned char stage[(CHUNK + PAD) * (sizeof(T) + 4)];
+    T* sval = reinterpret_cast<T*>(stage);
+    int32_t* scol = reinterpret_cast<int32_t*>(stage + (CHUNK + PAD) * sizeof(T));
     __shared__ int32_t srp[ROWS + 1];
     __shared__ double sred[NT / 32];
 
@@ -244,6 +629,18 @@ k_spmv_step(const StepArgs<T> a) {
     // now; everything up to griddepcontrol.wait reads only the matrix, which
     // no step writes, so it overlaps the previous step's tail.
     asm volatile("griddepcontrol.launch_dependents;");
+    if constexpr (DG) {
+        if (__ldg(a.diag.head) == 0) {   // uniform over the grid
+            __shared__ __align__(16) DiagSlot slot[DIAG_MAX];
+            __shared__ uint64_t bar;
+            __shared__ int info[2];
+            double sq = 0.0;
+            diag_tile<T, OP, NT, RPT, (CHUNK + PAD) * 2>(a, (int32_t)row0, nrows, (float*)stage, slot,
+                                                        &bar, info, sq);
+            if constexpr (OP == OP_RESID) block_sq<NT>(sq, sred, a.part);
+            return;
+        }
+    }
     // the tile that a CTA half a resident wave later stages: its nonzero
     // range is read now, beside this tile's row pointers.  CTAs near the end
     // of the grid prefetch the matrix tiles at the start of the next step
@@ -358,17 +755,7 @@ k_spmv_step(const StepArgs<T> a) {
         const int t = tid + q * NT;
         if (t < nrows) step_epilogue<T, OP>(a, row0 + t, acc[q], e0[q], e1[q], e2[q], sq);
     }
-    if constexpr (OP == OP_RESID) {
-        // deterministic block reduction of ||r||^2
-        for (int off = 16; off > 0; off >>= 1) sq += __shfl_down_sync(0xffffffffu, sq, off);
-        if ((tid & 31) == 0) sred[tid >> 5] = sq;
-        __syncthreads();
-        if (tid == 0) {
-            double t = 0.0;
-            for (int w = 0; w < NT / 32; ++w) t += sred[w];
-            a.part[blockIdx.x] = t;
-        }
-    }
+    if constexpr (OP == OP_RESID) block_sq<NT>(sq, sred, a.part);
 }
 
 // Direct-read step: the same step, one row per thread, the row's matrix
@@ -599,11 +986,7 @@ static size_t set_l2_exact(int dev, size_t bytes) {
 // 4646 / 5604: up to about 48 MB the streamed part loses next to nothing.
 constexpr size_t kPartialL2 = (size_t)48 << 20;
 
-int keep_a_flag(int64_t n, int64_t nnz, int elem, int nvec, bool may_reserve,
-                int32_t* keep_rows) {
-    if (keep_rows) *keep_rows = 0;
-    const int dev = current_device();
-    if (dev < 0) return 0;
+static int l2_bytes(int dev) {
     int l2 = g_l2_bytes[dev].load(std::memory_order_relaxed);
     if (l2 == 0) {
         int v = 0;
@@ -614,10 +997,22 @@ int keep_a_flag(int64_t n, int64_t nnz, int elem, int nvec, bool may_reserve,
         g_l2_bytes[dev].store(v, std::memory_order_relaxed);
         l2 = v;
     }
+    return l2;
+}
+
+// a chain's matrix and vectors fit comfortably in L2
+static bool fits_l2(double bytes, int l2) { return bytes <= 0.8 * (double)l2; }
+
+int keep_a_flag(int64_t n, int64_t nnz, int elem, int nvec, bool may_reserve,
+                int32_t* keep_rows) {
+    if (keep_rows) *keep_rows = 0;
+    const int dev = current_device();
+    if (dev < 0) return 0;
+    const int l2 = l2_bytes(dev);
     if (l2 <= 0 || n <= 0) return 0;
     const double a_bytes = (double)nnz * (elem + 4) + 4.0 * (n + 1);
     const double bytes = a_bytes + (double)nvec * n * elem;
-    if (!(bytes <= 0.8 * (double)l2)) {
+    if (!fits_l2(bytes, l2)) {
         // streaming: a chain holds the nonzeros of its leading rows in a
         // set-aside of kPartialL2 (shrinking a larger one that an L2-resident
         // workload left: an unused 76 MB set-aside cost the 160^3 FP32 chains
@@ -648,7 +1043,7 @@ static int step_resident_ctas() {
     int v = cached[dev].load(std::memory_order_relaxed);
     if (v == 0) {
         int occ = 0, sms = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_spmv_step<T, OP_P_REAL, true>,
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_spmv_step<T, OP_P_REAL, true, false>,
                                                           step_threads<T>(), 0) != cudaSuccess ||
             occ < 1)
             occ = 1;
@@ -660,6 +1055,58 @@ static int step_resident_ctas() {
         cached[dev].store(v, std::memory_order_relaxed);
     }
     return v;
+}
+
+// The diagonal form is tried with at most as many diagonals as keep it below
+// the CSR's bytes (an entry without its column index), where the steps to come
+// repay building it: about two passes over the matrix, 60 us for 1e6 rows of
+// five entries and 160 us for 4.1e6 rows of seven.  Per step, CSR against
+// diagonals (one value per diagonal / values of their own):
+//   streamed from HBM, 160^3:     49 us   24.4 us / 34 us   (repaid by 14 steps)
+//   held in L2, 1001 x 997:       9.0 us   6.2 us / 7.0 us  (repaid by 30)
+//   held in L2, 301 x 299:        2.2 us   -      / 2.3 us
+// (a matrix held in L2 is bound by what its CTAs of 128 rows cost to launch,
+// about 1 ns each, which smaller matrices do not feel).
+constexpr int64_t DIAG_MIN_STEPS = 20, DIAG_MIN_STEPS_L2 = 32;
+constexpr int32_t DIAG_MIN_ROWS_L2 = 700000;
+
+int32_t DiagStore::build(const int32_t* rowptr, const int32_t* colind, const float* vals, int32_t n,
+                         int64_t nnz, int64_t steps, cudaStream_t stream) {
+    if (n <= DIRECT_MAX_N || n > (1 << 30) || steps < DIAG_MIN_STEPS || nnz < n) return PPG_OK;
+    const int dev = current_device();
+    if (dev < 0) return PPG_OK;
+    if (fits_l2(8.0 * nnz + 16.0 * n, l2_bytes(dev)) &&
+        (n < DIAG_MIN_ROWS_L2 || steps < DIAG_MIN_STEPS_L2))
+        return PPG_OK;
+    const double avg = (double)nnz / (double)n;
+    const int most = (int)std::min<double>(DIAG_MAX, 2.0 * avg + 0.5);
+    if (avg > most) return PPG_OK;
+    const int32_t ld = (n + DIAG_PAD - 1) / DIAG_PAD * DIAG_PAD;
+    f.mask_bytes = most <= 8 ? 1 : most <= 16 ? 2 : 4;
+    const size_t b_vals = (size_t)most * ld * sizeof(float);
+    if (cudaMallocAsync(&mem, 1024 + b_vals + (size_t)ld * f.mask_bytes, stream) != cudaSuccess) {
+        cudaGetLastError();   // the CSR steps need none of it
+        mem = nullptr;
+        return PPG_OK;
+    }
+    static_assert(sizeof(DiagHead) <= 768, "the head's place");
+    s = stream;
+    char* m = (char*)mem;
+    DiagHead* H = (DiagHead*)m;
+    f.same = (const float*)(m + 768);
+    f.vals = (const float*)(m + 1024);
+    f.mask = m + 1024 + b_vals;
+    f.ld = ld;
+    k_diag_init<<<1, 64, 0, stream>>>(H);
+    k_diag_find<<<(n + DIAG_ROWS - 1) / DIAG_ROWS, DIAG_ROWS, 0, stream>>>(rowptr, colind, vals, n,
+                                                                           most, H);
+    k_diag_fill<<<(n + 255) / 256, 256, 0, stream>>>(rowptr, colind, vals, n, most, H, (float*)f.same,
+                                                        (float*)f.vals, ld, (void*)f.mask, f.mask_bytes);
+    g_launches += 3;
+    PPG_TRY(check_launch("k_diag_fill"));
+    f.head = H->w;
+    fresh = true;
+    return PPG_OK;
 }
 
 template <typename T, int PRE, int MINB, bool HINT>
@@ -681,16 +1128,16 @@ static cudaError_t launch_direct(cudaLaunchConfig_t& cfg, int op, const StepArgs
     }
 }
 
-template <typename T, bool PF>
+template <typename T, bool PF, bool DG>
 static cudaError_t launch_op(cudaLaunchConfig_t& cfg, int op, const StepArgs<T>& a) {
     switch (op) {
-        case OP_SPMV: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_SPMV, PF>, a);
-        case OP_RESID: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_RESID, PF>, a);
-        case OP_PHI_REAL: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_PHI_REAL, PF>, a);
-        case OP_PHI_PAIR2: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_PHI_PAIR2, PF>, a);
-        case OP_P_REAL: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_P_REAL, PF>, a);
-        case OP_P_PAIR1: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_P_PAIR1, PF>, a);
-        case OP_P_PAIR2: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_P_PAIR2, PF>, a);
+        case OP_SPMV: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_SPMV, PF, DG>, a);
+        case OP_RESID: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_RESID, PF, DG>, a);
+        case OP_PHI_REAL: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_PHI_REAL, PF, DG>, a);
+        case OP_PHI_PAIR2: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_PHI_PAIR2, PF, DG>, a);
+        case OP_P_REAL: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_P_REAL, PF, DG>, a);
+        case OP_P_PAIR1: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_P_PAIR1, PF, DG>, a);
+        case OP_P_PAIR2: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_P_PAIR2, PF, DG>, a);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -716,10 +1163,12 @@ int32_t launch_step(int op, const StepArgs<T>& a_in, cudaStream_t s) {
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = (a.flags & F_SERIAL) ? 0 : 1;
     if (op < OP_SPMV || op > OP_P_PAIR2) return PPG_ERR_ARG;
     const bool small = a_in.n <= DIRECT_MAX_N;
-    if (small || (a_in.flags & F_KEEP_A)) {
+    constexpr bool F32 = sizeof(T) == 4;
+    const bool dg = F32 && a.diag.head != nullptr;
+    if (small || ((a_in.flags & F_KEEP_A) && !dg)) {
         // one row per thread, no staging round (small system, or matrix in L2)
         const int dgrid = (int)(((int64_t)a_in.n + SPMV_ROWS - 1) / SPMV_ROWS);
         cfg.gridDim = dim3(dgrid);
@@ -769,7 +1218,7 @@ int32_t launch_step(int op, const StepArgs<T>& a_in, cudaStream_t s) {
         return rcd < 0 ? rcd : dgrid;
     }
     const cudaError_t e =
-        a.pf_ahead > 0 ? launch_op<T, true>(cfg, op, a) : launch_op<T, false>(cfg, op, a);
+        dg ? launch_op<T, true, F32>(cfg, op, a) : launch_op<T, true, false>(cfg, op, a);
     ++g_launches;
     if (e != cudaSuccess) {
         set_cuda_error(e, "cudaLaunchKernelEx(k_spmv_step)");
