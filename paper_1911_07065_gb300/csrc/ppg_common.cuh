@@ -174,6 +174,10 @@ struct StepArgs {
 // time of a step that is a handful of CTAs); the results are identical.
 constexpr int32_t DIRECT_MAX_N = 32768;
 
+// Rows of more entries than this are summed by a warp, in one order in every
+// kernel of the step (long_rows in spmv_root.cu), the others entry by entry.
+constexpr int32_t LONG_ROW = 128;
+
 // launch one fused step; returns the number of blocks (= partial sums for
 // OP_RESID) or a negative status
 template <typename T>

@@ -459,12 +459,15 @@ int32_t ppg_sweep_plan_create(const ppg_csr* A, const int32_t* perm_host, int32_
     P->halo_total = (int64_t)hidx.size();
     PPG_CUDA(cudaGetDevice(&P->dev));
     // fuse when the halo is at most 60 % of the rows (beyond that the
-    // redundant phase-A rows eat the saving) and the tile fits in shared
-    // memory
+    // redundant phase-A rows eat the saving), the tile fits in shared memory
+    // and no row is one of those that the plain step sums by a warp (this
+    // kernel sums every row in stored order)
+    int32_t max_len = 0;
+    for (int32_t i = 0; i < n; ++i) max_len = std::max(max_len, rp[i + 1] - rp[i]);
     int smem_max = 0;
     PPG_CUDA(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, P->dev));
     const size_t need = sweep_smem(T, max_halo);
-    P->fused = (fuse != 0 && (double)P->halo_total <= 0.6 * (double)n &&
+    P->fused = (fuse != 0 && max_len <= LONG_ROW && (double)P->halo_total <= 0.6 * (double)n &&
                 need <= (size_t)smem_max) ? 1 : 0;
     // one device allocation, owned by the plan
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
