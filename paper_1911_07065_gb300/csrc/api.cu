@@ -141,6 +141,7 @@ static int32_t run_steps(const std::vector<Step>& plan, int i0, int i1, const in
     double bytes = 0.0;
     int32_t keep_rows = 0;
     const int keep = keep_a_flag(n, nnz, (int)sizeof(T), 3, reserve_l2, &keep_rows);
+    const int sms = device_sm_count();
     for (int i = i0; i < i1; ++i) {
         const Step& st = plan[(size_t)i];
         if (st.op == OP_AXPY) {
@@ -165,6 +166,7 @@ static int32_t run_steps(const std::vector<Step>& plan, int i0, int i1, const in
         a.c2 = (T)st.c2;
         a.c3 = (T)st.c3;
         a.flags = st.flags | keep;
+        a.sms = sms;
         a.keep_rows = keep_rows;
         a.part = nullptr;
         if (diag) diag->give(a);

@@ -129,6 +129,7 @@ enum StepFlag : int {
     F_KEEP_A = 8,  // copy A with an L2 evict-last hint (A and the vectors fit in L2)
     F_SERIAL = 16, // not a programmatic dependent: the first step that reads a
                    // diagonal form built by the kernel before it
+    F_WIDE = 32,   // more than 5.5 entries in the average row
 };
 
 // An FP32 matrix by its diagonals (spmv_root.cu), built on the device inside
@@ -166,6 +167,7 @@ struct StepArgs {
     int32_t keep_rows;  // rows [0, keep_rows) stage their nonzeros with an L2
                         // evict-last hint (a chain over a matrix too large
                         // for L2 keeps its leading rows resident)
+    int32_t sms;        // the device's SMs (host side; 0: not looked up yet)
     DiagForm diag;      // FP32: the same matrix by diagonals (diag.head != nullptr)
 };
 
@@ -188,7 +190,8 @@ int32_t launch_step(int op, const StepArgs<T>& a, cudaStream_t s);
 template <typename T>
 int32_t launch_ew_step(int op, const StepArgs<T>& a, const T* prodv, cudaStream_t s);
 
-// F_KEEP_A when the matrix plus `nvec` work vectors fit comfortably in L2.
+// F_KEEP_A when the matrix plus `nvec` work vectors fit comfortably in L2
+// (with F_WIDE where its rows are that long).
 // The first such request reserves an L2 set-aside for the matrix (a limit of
 // the process's context on the current device); with may_reserve = false
 // nothing is reserved and F_KEEP_A is returned only if a set-aside large

@@ -802,12 +802,11 @@ k_spmv_step(const StepArgs<T> a) {
 // chain of a step is row pointers -> (wait) -> gathers -> epilogue.  Each
 // row is summed in stored order with one FMA per nonzero and the same
 // epilogue as k_spmv_step: bit-identical results.  Two uses:
-// * small systems (PRE = 8, no register bound, CTAs of DIRECT_SMALL_ROWS
-//   rows): a step is a handful of CTAs, and latency, not bytes, sets its
-//   time;
-// * a matrix held in L2 (F_KEEP_A; PRE = 3 or 4 and 32 registers, 8 CTAs
-//   per SM; the preloads carry the evict-last hint): the staging round trip
-//   is then the longer path.  2-D 1000^2 FP64 chains 57.3 -> 55.2 ms.
+// * small systems (PRE = 8, no register bound): a step is a handful of CTAs,
+//   and latency, not bytes, sets its time;
+// * a matrix held in L2 (F_KEEP_A; the preloads carry the evict-last hint):
+//   the staging round trip is then the longer path.  2-D 1000^2 FP64 chains
+//   57.3 -> 55.2 ms.  launch_step chooses PRE and the registers.
 // MINB: minimum CTAs per SM given to __launch_bounds__ (0: no register bound).
 // One row per thread of any CTA size up to SPMV_ROWS; the residual's partial
 // sums are one per CTA.
@@ -832,8 +831,8 @@ __device__ __forceinline__ int32_t ld_hint<int32_t>(const int32_t* p, uint64_t p
     return v;
 }
 
-constexpr int DIRECT_SMALL_ROWS = 64;   // rows (threads) per CTA for small systems
-constexpr int DIRECT_L2_ROWS = 128;     // ... and for a matrix held in L2
+constexpr int DIRECT_SMALL_ROWS = 64;   // rows (threads) per CTA, up to one such CTA per SM
+constexpr int DIRECT_L2_ROWS = 128;     // ... above that
 
 template <typename T, int OP, int PRE, int MINB, bool HINT>
 __global__ void __launch_bounds__(SPMV_ROWS, MINB)
@@ -1065,12 +1064,13 @@ int keep_a_flag(int64_t n, int64_t nnz, int elem, int nvec, bool may_reserve,
         return 0;
     }
     const size_t need = (size_t)(a_bytes * 1.05);
+    const int wide = (double)nnz > 5.5 * (double)n ? F_WIDE : 0;
     if (may_reserve) {
         reserve_l2_for(dev, need);
-        return F_KEEP_A;
+        return F_KEEP_A | wide;
     }
     // no change to the context: the hint only where a set-aside exists
-    return g_l2_reserved[dev].load(std::memory_order_relaxed) >= need ? F_KEEP_A : 0;
+    return g_l2_reserved[dev].load(std::memory_order_relaxed) >= need ? F_KEEP_A | wide : 0;
 }
 
 // CTAs of the root-step kernel resident at once (occupancy x SMs), per
@@ -1149,21 +1149,56 @@ int32_t DiagStore::build(const int32_t* rowptr, const int32_t* colind, const flo
     return PPG_OK;
 }
 
+// Even placement of a grid of a few CTAs per SM.  Launched as programmatic
+// dependents, the next steps' CTAs take their places before a step's own are
+// done, wherever there is room, and a step then starts with two CTAs on some
+// SMs and none on others.  Dynamic shared memory that nothing uses leaves each
+// SM room for its share alone: 40 FP64 steps on a grid of 150^2 156 -> 83 us,
+// 240^2 174 -> 88 us, 400^2 185 -> 148 us, on 30^3 159 -> 83 us.  It takes the
+// room from L1, so not above EVEN_MAX CTAs per SM (512^2, 14 per SM: 198 -> 205
+// us), and a grid of at most one CTA per SM needs none of it (50^2: 82 -> 87 us).
+constexpr int EVEN_MAX = 10;
+static size_t even_smem(unsigned grid, int sms, int most) {
+    const int per = (int)((grid + sms - 1) / sms);
+    if (per < 2 || per > most) return 0;
+    // 228 KB per SM, 1 KB of it taken by each CTA beside its own; a share and
+    // one CTA more must not fit
+    return (size_t)(228 / per - 2) * 1024;
+}
+
+template <typename T, int OP, int PRE, int MINB, bool HINT>
+static cudaError_t launch_even(cudaLaunchConfig_t& cfg, const StepArgs<T>& a, int most) {
+    auto kernel = k_spmv_direct<T, OP, PRE, MINB, HINT>;
+    static std::atomic<uint64_t> allowed{0};   // devices on which it may have more than 48 KB
+    size_t smem = even_smem(cfg.gridDim.x, a.sms, most);
+    if (smem > 48 * 1024) {
+        const int dev = current_device();
+        const uint64_t bit = dev < 0 ? 0 : 1ull << dev;
+        if (!(allowed.load(std::memory_order_relaxed) & bit)) {
+            if (dev >= 0 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 112 * 1024) == cudaSuccess) {
+                allowed.fetch_or(bit, std::memory_order_relaxed);
+            } else {
+                cudaGetLastError();
+                smem = 0;
+            }
+        }
+    }
+    cfg.dynamicSmemBytes = smem;
+    return cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
+// most: CTAs per SM up to which they are placed evenly (0: as they come)
 template <typename T, int PRE, int MINB, bool HINT>
-static cudaError_t launch_direct(cudaLaunchConfig_t& cfg, int op, const StepArgs<T>& a) {
+static cudaError_t launch_direct(cudaLaunchConfig_t& cfg, int op, const StepArgs<T>& a, int most) {
     switch (op) {
-        case OP_SPMV: return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_SPMV, PRE, MINB, HINT>, a);
-        case OP_RESID: return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_RESID, PRE, MINB, HINT>, a);
-        case OP_PHI_REAL:
-            return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_PHI_REAL, PRE, MINB, HINT>, a);
-        case OP_PHI_PAIR2:
-            return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_PHI_PAIR2, PRE, MINB, HINT>, a);
-        case OP_P_REAL:
-            return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_P_REAL, PRE, MINB, HINT>, a);
-        case OP_P_PAIR1:
-            return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_P_PAIR1, PRE, MINB, HINT>, a);
-        case OP_P_PAIR2:
-            return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_P_PAIR2, PRE, MINB, HINT>, a);
+        case OP_SPMV: return launch_even<T, OP_SPMV, PRE, MINB, HINT>(cfg, a, most);
+        case OP_RESID: return launch_even<T, OP_RESID, PRE, MINB, HINT>(cfg, a, most);
+        case OP_PHI_REAL: return launch_even<T, OP_PHI_REAL, PRE, MINB, HINT>(cfg, a, most);
+        case OP_PHI_PAIR2: return launch_even<T, OP_PHI_PAIR2, PRE, MINB, HINT>(cfg, a, most);
+        case OP_P_REAL: return launch_even<T, OP_P_REAL, PRE, MINB, HINT>(cfg, a, most);
+        case OP_P_PAIR1: return launch_even<T, OP_P_PAIR1, PRE, MINB, HINT>(cfg, a, most);
+        case OP_P_PAIR2: return launch_even<T, OP_P_PAIR2, PRE, MINB, HINT>(cfg, a, most);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -1213,49 +1248,54 @@ int32_t launch_step(int op, const StepArgs<T>& a_in, cudaStream_t s) {
         const int dgrid = (int)(((int64_t)a_in.n + SPMV_ROWS - 1) / SPMV_ROWS);
         cfg.gridDim = dim3(dgrid);
         cfg.blockDim = dim3(SPMV_ROWS);
-        // matrix in L2: entries preloaded before the dependency wait -- four
-        // at 32 registers (2048 threads per SM), five for the plain SpMV step
-        // (still 32), five at 40 registers (1536 threads) for the second step
-        // of a pair of Algorithm 1, which spills at 32 (2-D 1000^2 FP64
-        // chains: staged kernel 57.3 ms; direct with four preloads 55.8 ms
-        // (without the evict-last hint 56.3 ms); three for the pair step at
-        // 32 registers 55.2 ms; with 128-row CTAs 54.7 ms; five for the plain
-        // SpMV step 53.4 ms; five for the pair step at 40 registers 52.5 ms,
-        // four there 52.8 ms)
-        cudaError_t ed;
-        if (small) {
-            // 64-row CTAs (the residual keeps 256: one partial sum per 256
-            // rows): a small system's step then spreads over 4x the SMs
-            // (2-D 50^2 p(A) v 37.9 -> 32.7 us; 128 rows 35.6, 32 rows 36.8;
-            // 100^2 56.1 -> 49.5 us)
-            if (op != OP_RESID) {
-                cfg.blockDim = dim3(DIRECT_SMALL_ROWS);
-                cfg.gridDim = dim3((unsigned)(((int64_t)a_in.n + DIRECT_SMALL_ROWS - 1) /
-                                              DIRECT_SMALL_ROWS));
-            }
-            ed = launch_direct<T, 8, 0, false>(cfg, op, a);
-        } else {
-            // matrix in L2: 128-row CTAs (2-D 1000^2 FP64 chains 55.22 ->
-            // 54.88 ms against 256 rows; 64 rows 69.5 ms)
-            if (op != OP_RESID) {
-                cfg.blockDim = dim3(DIRECT_L2_ROWS);
-                cfg.gridDim = dim3((unsigned)(((int64_t)a_in.n + DIRECT_L2_ROWS - 1) /
-                                              DIRECT_L2_ROWS));
-            }
-            if (op == OP_PHI_PAIR2)   // five entries at 40 registers
-                ed = launch_direct<T, 5, 6, true>(cfg, op, a);
-            else if (op == OP_SPMV)   // five entries: a 5-point row whole
-                ed = launch_direct<T, 5, 8, true>(cfg, op, a);
-            else
-                ed = launch_direct<T, 4, 8, true>(cfg, op, a);
+        // CTAs of 64 rows while an SM each is enough (a step then spreads over
+        // more of them: 2-D 50^2 p(A) v 37.9 -> 32.7 us against 256 rows; 128
+        // rows 35.6, 32 rows 36.8), else of 128 (1000^2 FP64 chains 55.22 ->
+        // 54.88 ms against 256 rows; 64 rows 69.5 ms); the residual keeps 256:
+        // one partial sum per 256 rows
+        const int sms = a.sms = a.sms ? a.sms : device_sm_count();
+        if (op != OP_RESID) {
+            const int rows_d = a_in.n <= sms * DIRECT_SMALL_ROWS ? DIRECT_SMALL_ROWS : DIRECT_L2_ROWS;
+            cfg.blockDim = dim3(rows_d);
+            cfg.gridDim = dim3((unsigned)(((int64_t)a_in.n + rows_d - 1) / rows_d));
         }
+        const int most = op == OP_RESID ? 0 : EVEN_MAX;
+        // matrix in L2: entries preloaded before the dependency wait.
+        // Up to 5.5 in the average row, FP64: four at 32 registers (2048
+        // threads per SM), five for the plain SpMV step (still 32), five at 40
+        // registers (1536 threads) for the second step of a pair of Algorithm
+        // 1, which spills at 32 (2-D 1000^2 FP64 chains: staged kernel 57.3 ms;
+        // direct with four preloads 55.8 ms (without the evict-last hint 56.3
+        // ms); three for the pair step at 32 registers 55.2 ms; with 128-row
+        // CTAs 54.7 ms; five for the plain SpMV step 53.4 ms; five for the pair
+        // step at 40 registers 52.5 ms, four there 52.8 ms).  FP32: five at 40
+        // registers throughout (40 steps: 400^2 105 -> 94 us, 512^2 137 -> 124
+        // us, 700^2 194 -> 184 us; FP64 700^2 295 -> 298 us).
+        // Above, a seven-entry row whole at 40 registers (FP64 60 x 70 x 80 phi
+        // chains of 40 295 -> 268 us, FP32 p chains of 20 100 -> 79 us; 48
+        // registers 279 and 80 us, six entries 287 and 88 us), and eight at 64
+        // registers in FP64 while those 8 CTAs per SM hold the whole matrix
+        // (45^3 201 -> 137 us, seven 146 us; 53^3 247 -> 168 us, seven 203 us).
+        cudaError_t ed;
+        if (small)
+            ed = launch_direct<T, 8, 0, false>(cfg, op, a, most);
+        else if ((a_in.flags & F_WIDE) && !F32 && a_in.n <= sms * 8 * DIRECT_L2_ROWS)
+            ed = launch_direct<T, 8, 4, true>(cfg, op, a, min(most, 6));   // (above, registers do it)
+        else if (a_in.flags & F_WIDE)
+            ed = launch_direct<T, 7, 6, true>(cfg, op, a, most);
+        else if (F32 || op == OP_PHI_PAIR2)
+            ed = launch_direct<T, 5, 6, true>(cfg, op, a, most);
+        else if (op == OP_SPMV)
+            ed = launch_direct<T, 5, 8, true>(cfg, op, a, most);
+        else
+            ed = launch_direct<T, 4, 8, true>(cfg, op, a, most);
         ++g_launches;
         if (ed != cudaSuccess) {
             set_cuda_error(ed, "cudaLaunchKernelEx(k_spmv_direct)");
+            cudaGetLastError();
             return PPG_ERR_CUDA;
         }
-        const int32_t rcd = check_launch("k_spmv_direct");
-        return rcd < 0 ? rcd : dgrid;
+        return dgrid;
     }
     const cudaError_t e =
         dg ? launch_op<T, true, F32>(cfg, op, a) : launch_op<T, true, false>(cfg, op, a);
