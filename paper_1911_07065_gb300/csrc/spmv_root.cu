@@ -1156,14 +1156,15 @@ int32_t DiagStore::build(const int32_t* rowptr, const int32_t* colind, const flo
 // SM room for its share alone: 40 FP64 steps on a grid of 150^2 156 -> 83 us,
 // 240^2 174 -> 88 us, 400^2 185 -> 148 us, on 30^3 159 -> 83 us.  It takes the
 // room from L1, so not above EVEN_MAX CTAs per SM (512^2, 14 per SM: 198 -> 205
-// us), and a grid of at most one CTA per SM needs none of it (50^2: 82 -> 87 us).
+// us), and a grid of no more CTAs than half the SMs needs none of it (50^2: 82 -> 87
+// us).
 constexpr int EVEN_MAX = 10;
 static size_t even_smem(unsigned grid, int sms, int most) {
     const int per = (int)((grid + sms - 1) / sms);
-    if (per < 2 || per > most) return 0;
+    if (per > most || 2 * grid <= (unsigned)sms) return 0;
     // 228 KB per SM, 1 KB of it taken by each CTA beside its own; a share and
     // one CTA more must not fit
-    return (size_t)(228 / per - 2) * 1024;
+    return (size_t)min(228 / per - 2, 116) * 1024;
 }
 
 template <typename T, int OP, int PRE, int MINB, bool HINT>
@@ -1176,7 +1177,7 @@ static cudaError_t launch_even(cudaLaunchConfig_t& cfg, const StepArgs<T>& a, in
         const uint64_t bit = dev < 0 ? 0 : 1ull << dev;
         if (!(allowed.load(std::memory_order_relaxed) & bit)) {
             if (dev >= 0 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 112 * 1024) == cudaSuccess) {
+                                                 116 * 1024) == cudaSuccess) {
                 allowed.fetch_or(bit, std::memory_order_relaxed);
             } else {
                 cudaGetLastError();
