@@ -139,6 +139,16 @@ static int32_t run_steps(const std::vector<Step>& plan, int i0, int i1, const in
                          const Buffers& bufs, cudaStream_t s, double* bytes_out,
                          bool reserve_l2, DiagStore* diag) {
     double bytes = 0.0;
+    if (i0 == i1) {
+        if (bytes_out) *bytes_out = 0.0;
+        return PPG_OK;
+    }
+    if (i0 == 0 && i1 == (int)plan.size() && chain_cluster_fits<T>(plan, n, nnz)) {
+        PPG_TRY(launch_chain_cluster<T>(plan, rowptr, colind, vals, n, bufs, s));
+        for (const Step& st : plan) bytes += step_bytes(st.op, st.flags, n, nnz, (int)sizeof(T));
+        if (bytes_out) *bytes_out = bytes;
+        return PPG_OK;
+    }
     int32_t keep_rows = 0;
     const int keep = keep_a_flag(n, nnz, (int)sizeof(T), 3, reserve_l2, &keep_rows);
     const int sms = device_sm_count();
@@ -586,7 +596,13 @@ static int32_t run_solve(SolveCore& c) {
     constexpr int kLookahead = 2;
     const std::vector<Step>* chain = pp ? (c.flex ? &c.p_plan : &c.phi_plan) : nullptr;
     // (the fused-sweep chain runs whole: its pairs must not be split)
-    const int nahead = (chain && !c.sweep)
+    // (a chain that is one launch goes ahead whole: its result, basis column
+    // j + 2, is not read by the update either)
+    const bool whole = chain && !c.sweep &&
+                       (c.flex ? chain_cluster_fits<float>(*chain, n, nnz)
+                               : chain_cluster_fits<double>(*chain, n, nnz));
+    const int nahead = whole ? (int)chain->size()
+                       : (chain && !c.sweep)
                            ? std::max(0, std::min(kLookahead, (int)chain->size() - 1))
                            : 0;
     auto chain_steps = [&](int j, int i0, int i1, double* by) -> int32_t {
