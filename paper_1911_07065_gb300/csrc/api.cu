@@ -353,6 +353,21 @@ static int32_t cgs2_column(SolveCore& c, int j, double* w, bool with_self, Event
     return PPG_OK;
 }
 
+// Arnoldi step j after the operator product w: CGS2, the Hessenberg column (with
+// its rotation when givens) and, where that comes in the same launch, the
+// scaling of w (*scaled).
+static int32_t orthogonalise(SolveCore& c, int ldh, int j, double* w, bool with_self, bool givens,
+                             double bnorm, double brtol, EventPair* ev, bool* scaled) {
+    *scaled = !c.opts.cgs2_fused && arnoldi_small_fits(c.A64->n, j + 1);
+    if (*scaled) {
+        if (ev) ev->start(c.s);
+        return launch_arnoldi_small(c.V, c.ldv, j, w, c.A64->n, with_self, c.gs, ldh, givens, bnorm, brtol,
+                                    c.s);
+    }
+    PPG_TRY(cgs2_column(c, j, w, with_self, ev));
+    return launch_finish_column(c.gs, ldh, j, c.ows.h1, c.ows.h2, c.ows.nrm, givens, bnorm, brtol, c.s);
+}
+
 // the error flag of the fused CGS2 pass (a staging wait gave up); `flag`
 // is host memory filled by a copy the caller has synchronised
 static int32_t ortho_status(const unsigned* flag) {
@@ -426,10 +441,9 @@ static int32_t build_core(const ppg_csr* A, int d, const double* v0, const ppg_o
             int32_t g = launch_step<double>(OP_SPMV, a, s);
             if (g < 0) return g;
         }
-        PPG_TRY(cgs2_column(c, j, w, true, nullptr));
-        PPG_TRY(launch_finish_column(c.gs, ldh, j, c.ows.h1, c.ows.h2, c.ows.nrm, false, 1.0,
-                                     1e-13, s));
-        PPG_TRY(launch_scale(w, w, n, c.gs.scal + 2, s));
+        bool scaled = false;
+        PPG_TRY(orthogonalise(c, ldh, j, w, true, false, 1.0, 1e-13, nullptr, &scaled));
+        if (!scaled) PPG_TRY(launch_scale(w, w, n, c.gs.scal + 2, s));
     }
     std::vector<double> H((size_t)ldh * d), sc(8);
     PPG_CUDA(cudaMemcpyAsync(H.data(), c.gs.Hraw, sizeof(double) * ldh * d,
@@ -647,6 +661,7 @@ static int32_t run_solve(SolveCore& c) {
         return PPG_OK;
     };
     // the rest of step j from chain step `from` on
+    bool scaled = false;   // basis column j + 1 has its scale
     auto finish_step = [&](int j, int e, int from, double* by) -> int32_t {
         double* vj = c.V + (size_t)j * c.ldv;
         double* w = c.V + (size_t)(j + 1) * c.ldv;
@@ -684,9 +699,7 @@ static int32_t run_solve(SolveCore& c) {
             ev_poly[e].stop(s);
             *by = step_bytes(OP_SPMV, 0, n, nnz, 8);
         }
-        PPG_TRY(cgs2_column(c, j, w, false, &ev_orth[e]));
-        PPG_TRY(launch_finish_column(c.gs, ldh, j, c.ows.h1, c.ows.h2, c.ows.nrm, true, bnorm,
-                                     0.0, s));
+        PPG_TRY(orthogonalise(c, ldh, j, w, false, true, bnorm, 0.0, &ev_orth[e], &scaled));
         ev_orth[e].stop(s);
         PPG_CUDA(cudaMemcpyAsync(scal_h, c.gs.scal, 4 * sizeof(double), cudaMemcpyDeviceToHost,
                                  s));
@@ -709,7 +722,7 @@ static int32_t run_solve(SolveCore& c) {
             const double by_step = by_cur;
             from = 0;
             if (j + 1 < m) {   // look-ahead into step j + 1
-                PPG_TRY(launch_scale(w, w, n, c.gs.scal + 2, s));
+                if (!scaled) PPG_TRY(launch_scale(w, w, n, c.gs.scal + 2, s));
                 PPG_TRY(begin_step(j + 1, e ^ 1, nahead, &by_cur));
                 from = nahead;
             }

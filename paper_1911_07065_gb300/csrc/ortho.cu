@@ -661,66 +661,107 @@ int32_t launch_cgs_sub_dot(const double* V, int64_t ldv, int ncol, double* w, in
 // Hessenberg column, Givens rotation, shortcut residual (one thread)
 // ---------------------------------------------------------------------------
 
-__global__ void k_finish_column(GmresState st, int ldh, int j, const double* h1,
-                                const double* h2, const double* nrm, int givens,
-                                double bnorm, double brtol) {
-    // one warp stages the column and the rotations in shared memory, then
-    // one thread applies the j earlier rotations and makes the new one
-    __shared__ double col[ORTHO_MAXC + 1];
-    __shared__ double scs[ORTHO_MAXC], ssn[ORTHO_MAXC];
-    const int lane = threadIdx.x;
-    PPG_PDL_TRIGGER();
-    PPG_PDL_WAIT();
-    for (int i = lane; i <= j; i += 32) col[i] = h1[i] + h2[i];
-    if (givens)
-        for (int i = lane; i < j; i += 32) {
-            scs[i] = st.cs[i];
-            ssn[i] = st.sn[i];
+// The Hessenberg column is one warp's work and a chain of FP64 operations, about
+// 80 cycles each for a warp whether one lane or all take part, so what can go
+// side by side goes into lanes: the products of the earlier rotations, which
+// leave one FMA per rotation in the chain, then the three square roots in one
+// and the four divisions in one.  One lane doing all of it took 4,600 + 300 j
+// cycles, with every solve below 10,000 rows 4 % slower.
+
+struct ColumnSmem {
+    double col[ORTHO_MAXC + 1], cs[ORTHO_MAXC], sn[ORTHO_MAXC];
+    double p[ORTHO_MAXC], ci[ORTHO_MAXC + 1];
+};
+struct ColumnTop {
+    double a, gj, w0sq, flag;   // a: entry j after the earlier rotations
+};
+
+// what does not need the norm of the new vector
+__device__ __forceinline__ ColumnTop rotate_column(const GmresState& st, int ldh, int j, const double* h1,
+                                                   const double* h2, int givens, double brtol,
+                                                   ColumnSmem& m) {
+    const int lane = threadIdx.x & 31;
+    ColumnTop t{0.0, 0.0, 0.0, st.scal[5]};
+    if (brtol > 0.0) t.w0sq = h1[j + 1];   // ||A v_j||^2 from the first dot pass
+    for (int i = lane; i <= j; i += 32) {
+        const double v = h1[i] + h2[i];
+        m.col[i] = v;
+        if (st.Hraw) st.Hraw[(size_t)j * ldh + i] = v;
+    }
+    if (!givens) return t;
+    t.gj = st.g[j];
+    __syncwarp();
+    for (int i = lane; i < j; i += 32) {
+        const double c = st.cs[i];
+        m.cs[i] = c;
+        m.sn[i] = st.sn[i];
+        m.p[i] = c * m.col[i + 1];
+    }
+    __syncwarp();
+    if (lane == 0) {
+        double ci = m.col[0];
+#pragma unroll 4
+        for (int i = 0; i < j; ++i) {
+            m.ci[i] = ci;
+            ci = fma(-m.sn[i], ci, m.p[i]);
         }
-    const double hn = sqrt(fmax(nrm[0], 0.0));
-    if (lane == 0) col[j + 1] = hn;
+        m.ci[j] = ci;
+    }
     __syncwarp();
-    if (st.Hraw)
-        for (int i = lane; i <= j + 1; i += 32) st.Hraw[(size_t)j * ldh + i] = col[i];
-    __syncwarp();
+    for (int i = lane; i < j; i += 32)
+        st.R[(size_t)j * ldh + i] = m.cs[i] * m.ci[i] + m.sn[i] * m.col[i + 1];
+    t.a = m.ci[j];
+    return t;
+}
+
+// the rest, with nsq the square of that norm
+__device__ __forceinline__ void close_column(const GmresState& st, int ldh, int j, const ColumnTop& t,
+                                             double nsq, int givens, double bnorm, double brtol) {
+    const int lane = threadIdx.x & 31;
+    nsq = fmax(nsq, 0.0);
+    const double r2 = fma(t.a, t.a, nsq);
+    const double y = sqrt(lane == 0 ? nsq : lane == 1 ? fmax(t.w0sq, 0.0) : r2);
+    const double hn = __shfl_sync(0xffffffffu, y, 0);
+    const double w0 = __shfl_sync(0xffffffffu, y, 1);
+    double r = __shfl_sync(0xffffffffu, y, 2);
+    if (!(r2 > 1e-280 && r2 < 1e280)) r = hypot(t.a, hn);   // (squares out of range)
+    const double q = (lane == 0 ? 1.0 : lane == 1 ? t.a : lane == 2 ? hn : fabs(t.gj)) /
+                     (lane == 0 ? hn : lane == 3 ? bnorm : r);
+    double c = __shfl_sync(0xffffffffu, q, 1), s = __shfl_sync(0xffffffffu, q, 2);
+    const double gb = __shfl_sync(0xffffffffu, q, 3);
+    if (r == 0.0) {
+        c = 1.0;
+        s = 0.0;
+    }
     if (lane != 0) return;
     double* sc = st.scal;
-    bool brk;
-    if (brtol > 0.0) {
-        const double w0 = sqrt(fmax(h1[j + 1], 0.0));   // ||A v_j|| from the first dot pass
-        brk = !(hn > brtol * w0);
-    } else {
-        brk = !(hn > 0.0);
-    }
-    if (brk && sc[5] == 0.0) {
+    const bool brk = brtol > 0.0 ? !(hn > brtol * w0) : !(hn > 0.0);
+    if (brk && t.flag == 0.0) {
         sc[5] = 1.0;
         sc[6] = (double)j;
     }
-    if (brk && st.Hraw) st.Hraw[(size_t)j * ldh + j + 1] = 0.0;
+    if (st.Hraw) st.Hraw[(size_t)j * ldh + j + 1] = brk ? 0.0 : hn;
     sc[1] = hn;
-    sc[2] = (hn > 0.0 && !brk) ? 1.0 / hn : 0.0;
+    sc[2] = (hn > 0.0 && !brk) ? q : 0.0;
     if (givens) {
-        double ci = col[0];
-        for (int i = 0; i < j; ++i) {
-            const double nxt = col[i + 1];
-            const double t = scs[i] * ci + ssn[i] * nxt;
-            ci = -ssn[i] * ci + scs[i] * nxt;
-            col[i] = t;
-        }
-        col[j] = ci;
-        const double a = col[j], b = col[j + 1];
-        const double r = hypot(a, b);
-        double c = 1.0, s = 0.0;
-        if (r != 0.0) { c = a / r; s = b / r; }
         st.cs[j] = c;
         st.sn[j] = s;
-        col[j] = r;
-        for (int i = 0; i <= j; ++i) st.R[(size_t)j * ldh + i] = col[i];
-        const double gj = st.g[j];
-        st.g[j + 1] = -s * gj;
-        st.g[j] = c * gj;
-        sc[0] = fabs(st.g[j + 1]) / bnorm;
+        st.R[(size_t)j * ldh + j] = r;
+        st.g[j + 1] = -s * t.gj;
+        st.g[j] = c * t.gj;
+        sc[0] = fabs(s) * gb;
     }
+}
+
+__global__ void k_finish_column(GmresState st, int ldh, int j, const double* h1,
+                                const double* h2, const double* nrm, int givens,
+                                double bnorm, double brtol) {
+    __shared__ ColumnSmem m;
+    PPG_PDL_TRIGGER();
+    PPG_PDL_WAIT();
+    const double nsq = nrm[0];
+    const ColumnTop t = rotate_column(st, ldh, j, h1, h2, givens, brtol, m);
+    close_column(st, ldh, j, t, nsq, givens, bnorm, brtol);
 }
 
 int32_t launch_finish_column(const GmresState& st, int ldh, int j, const double* h1,
@@ -936,5 +977,315 @@ template int32_t launch_axpby<double>(double, const double*, double, const doubl
                                       double*, int32_t, cudaStream_t);
 template int32_t launch_axpby<float>(float, const float*, float, const float*, float*,
                                      int32_t, cudaStream_t);
+
+// ---------------------------------------------------------------------------
+// A small system's whole orthogonalisation step in one launch: CGS2 of w
+// against columns 0..j, the Hessenberg column with its rotation, and the
+// scaling of w, by one cluster of SMALL_CTAS CTAs.
+//
+// As launches of their own (two dot and two update passes, the column, the
+// scaling) these take 38 us at n = 2,500 one by one, for 0.2 us of HBM traffic:
+// each waits for the one before it and for a last CTA's sums.  Here a CTA keeps
+// its rows of w and of the basis in shared memory for all four passes, and the
+// CTAs exchange the partial sums through each other's shared memory between
+// cluster barriers.  40 Arnoldi steps at 1,600 rows take 0.83 ms, as launches of
+// their own 1.52, at 6,400 rows 1.13 and 1.62; a solve at 2,500 rows 0.88 and
+// 1.28.  FP64 arithmetic on SMALL_CTAS of the SMs ends its range
+// (arnoldi_small_fits).
+// ---------------------------------------------------------------------------
+
+constexpr int SMALL_CTAS = 16;
+constexpr int SMALL_THREADS = 512;          // and one more warp, for the Hessenberg column
+constexpr int SMALL_COLS = 64;              // columns at most
+constexpr size_t SMALL_SMEM = 190 * 1024;   // for a CTA's rows of w and V
+
+struct SmallArnoldi {
+    const double* V;
+    int64_t ldv;
+    double* w;
+    int32_t n, j, chunk, cached;   // rows per CTA; columns that fit
+    int32_t with_self, givens, ldh;
+    double bnorm, brtol;
+    GmresState st;
+};
+
+__device__ __forceinline__ double ld_rank(const double* own, uint32_t rank) {
+    uint32_t a;
+    double v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(own)), "r"(rank));
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void cluster_arrive() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_sync_all() {
+    cluster_arrive();
+    cluster_wait();
+}
+__device__ __forceinline__ void worker_sync() {
+    asm volatile("bar.sync 1, %0;" ::"n"(SMALL_THREADS) : "memory");
+}
+
+// each of v[0..3] summed over the lanes: lane 8 k has the total of value k (in
+// bit order 16, 8)
+__device__ __forceinline__ double warp_reduce4(double (&v)[4], int lane) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const bool hi = lane & 16;
+        const double send = hi ? v[i] : v[i + 2];
+        const double keep = hi ? v[i + 2] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+    }
+    const bool hi = lane & 8;
+    const double send = hi ? v[0] : v[1];
+    double r = (hi ? v[1] : v[0]) + __shfl_xor_sync(0xffffffffu, send, 8);
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) r += __shfl_xor_sync(0xffffffffu, r, off);
+    return r;
+}
+
+// dot products of columns c0..c0 + P - 1 (those below nv) with w over this CTA's rows
+template <int P, class F>
+__device__ __forceinline__ void small_dots(int c0, int nv, int rows, int lane, const F& column,
+                                           const double* ws, double* part) {
+    const double* col[P];
+#pragma unroll
+    for (int i = 0; i < P; ++i) col[i] = column(min(c0 + i, nv - 1));
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 2
+    for (int r = lane; r < rows; r += 32) {
+        const double x = ws[r];
+#pragma unroll
+        for (int i = 0; i < P; ++i) v[i] = fma(col[i][r], x, v[i]);
+    }
+    if (P == 1) {
+        const double t = warp_sum(v[0]);
+        if (lane == 0) part[c0] = t;
+    } else {
+        if (P == 2) {   // one value to each half warp
+            const bool hi = lane & 16;
+            double t = (hi ? v[1] : v[0]) + __shfl_xor_sync(0xffffffffu, hi ? v[0] : v[1], 16);
+#pragma unroll
+            for (int off = 8; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+            if ((lane & 15) == 0 && c0 + (lane >> 4) < nv) part[c0 + (lane >> 4)] = t;
+        } else {
+            const double t = warp_reduce4(v, lane);
+            const int k = lane >> 3;
+            if ((lane & 7) == 0 && c0 + k < nv) part[c0 + k] = t;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(SMALL_THREADS + 32, 1) k_arnoldi_small(const SmallArnoldi a) {
+    extern __shared__ __align__(16) double small_rows[];   // [chunk] of w, [cached][chunk] of V
+    __shared__ double s_part[2][SMALL_COLS + 2];
+    __shared__ double s_h[2][SMALL_COLS + 2];
+    __shared__ double s_half[SMALL_THREADS / 2];
+    __shared__ double s_red[SMALL_THREADS / 32];
+    __shared__ double s_inv;
+    __shared__ ColumnSmem s_col;
+    constexpr int NW = SMALL_THREADS / 32;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const bool worker = warp < NW;
+    uint32_t rank;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    const int64_t r0 = (int64_t)rank * a.chunk;
+    const int rows = (int)max((int64_t)0, min((int64_t)a.chunk, a.n - r0));
+    const int ncol = a.j + 1;
+    double* const ws = small_rows;
+    double* const Vs = small_rows + a.chunk;
+    PPG_PDL_TRIGGER();
+    PPG_PDL_WAIT();
+    if (worker) {
+        for (int r = tid; r < rows; r += SMALL_THREADS) ws[r] = a.w[r0 + r];
+        for (int c = warp; c < a.cached; c += NW)
+            for (int r = lane; r < rows; r += 32) Vs[c * a.chunk + r] = a.V[c * a.ldv + r0 + r];
+    }
+    __syncthreads();
+    auto column = [&](int c) -> const double* {
+        return c == ncol ? ws : c < a.cached ? Vs + c * a.chunk : a.V + c * a.ldv + r0;
+    };
+    // the sum over the CTAs of part[k]: four neighbouring lanes to a value, q the
+    // lane's number among them
+    auto cluster_sum = [&](const double* part, int k, int q) {
+        double v = 0.0;
+#pragma unroll
+        for (int i = 0; i < SMALL_CTAS / 4; ++i) v += ld_rank(part + k, q + 4 * i);
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        return v + __shfl_xor_sync(0xffffffffu, v, 2);
+    };
+    // Two CGS2 passes.  A CTA writes s_part[0] again, for the norm, only after
+    // the second pass's barrier, when all have read the first pass's values.
+    for (int pass = 0; pass < 2; ++pass) {
+        const int nv = ncol + (pass == 0 && a.with_self ? 1 : 0);
+        double* const part = s_part[pass];
+        double* const h = s_h[pass];
+        // columns to a warp: enough that four warps, one per scheduler, take all
+        // the columns, and up to four, where a warp's sums cost least
+        if (!worker) {
+        } else if (nv <= 4) {
+            if (warp < nv) small_dots<1>(warp, nv, rows, lane, column, ws, part);
+        } else if (nv <= 8) {
+            if (2 * warp < nv) small_dots<2>(2 * warp, nv, rows, lane, column, ws, part);
+        } else {
+            for (int c0 = 4 * warp; c0 < nv; c0 += 4 * NW)
+                small_dots<4>(c0, nv, rows, lane, column, ws, part);
+        }
+        cluster_sync_all();
+        if (warp * 8 < nv && worker) {
+            const int c = tid >> 2;
+            const double v = cluster_sum(part, min(c, nv - 1), tid & 3);
+            if (c < nv && (tid & 3) == 0) h[c] = v;
+        }
+        __syncthreads();
+        if (pass == 1 && !worker) break;
+        // w -= V h, even and odd columns by different warps where the rows leave room
+        if (2 * a.chunk <= SMALL_THREADS) {
+            const int half = tid >= a.chunk ? 1 : 0, r = tid - half * a.chunk;
+            double s = 0.0;
+            if (r < rows && worker) {
+                for (int c = half; c < ncol; c += 2) s = fma(column(c)[r], h[c], s);
+                if (half) s_half[r] = s;
+            }
+            if (pass == 0) __syncthreads();
+            else worker_sync();
+            if (!half && r < rows) ws[r] -= s + s_half[r];
+        } else if (worker) {
+            for (int r = tid; r < rows; r += SMALL_THREADS) {
+                double s = 0.0, s1 = 0.0;
+                int c = 0;
+                for (; c + 1 < ncol; c += 2) {
+                    s = fma(column(c)[r], h[c], s);
+                    s1 = fma(column(c + 1)[r], h[c + 1], s1);
+                }
+                if (c < ncol) s = fma(column(c)[r], h[c], s);
+                ws[r] -= s + s1;
+            }
+        }
+        if (pass == 0) __syncthreads();
+    }
+    if (!worker) {
+        // the column warp: CTA 0's turns the rotations while the others do the
+        // second update and the norm
+        cluster_arrive();
+        ColumnTop top{};
+        if (rank == 0) top = rotate_column(a.st, a.ldh, a.j, s_h[0], s_h[1], a.givens, a.brtol, s_col);
+        cluster_wait();
+        const double nsq = cluster_sum(s_part[0], 0, lane & 3);
+        cluster_arrive();
+        if (rank == 0) close_column(a.st, a.ldh, a.j, top, nsq, a.givens, a.bnorm, a.brtol);
+        cluster_wait();
+        return;
+    }
+    // ||w||^2: a thread's own rows, the ones it has just updated
+    double sq = 0.0;
+    for (int r = tid; r < rows; r += SMALL_THREADS) sq = fma(ws[r], ws[r], sq);
+    if (warp * 32 < rows) {
+        sq = warp_sum(sq);
+        if (lane == 0) s_red[warp] = sq;
+    }
+    worker_sync();
+    if (tid == 0) {
+        double t = 0.0;
+        const int nw = min(NW, (rows + 31) / 32);
+        for (int k = 0; k < nw; ++k) t += s_red[k];
+        s_part[0][0] = t;
+    }
+    cluster_sync_all();
+    if (warp == 0) {
+        const double nsq = cluster_sum(s_part[0], 0, lane & 3);
+        // as close_column decides it
+        const double y = sqrt(fmax(lane == 1 && a.brtol > 0.0 ? s_h[0][ncol] : nsq, 0.0));
+        const double hn = __shfl_sync(0xffffffffu, y, 0), w0 = __shfl_sync(0xffffffffu, y, 1);
+        const bool brk = a.brtol > 0.0 ? !(hn > a.brtol * w0) : !(hn > 0.0);
+        if (lane == 0) s_inv = (hn > 0.0 && !brk) ? 1.0 / hn : 0.0;
+    }
+    worker_sync();
+    cluster_arrive();   // (done with the others' memory)
+    const double inv = s_inv;
+    for (int r = tid; r < rows; r += SMALL_THREADS) a.w[r0 + r] = ws[r] * inv;
+    cluster_wait();
+}
+
+static int32_t small_launch(const SmallArnoldi& a, size_t smem, bool probe, int* clusters, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(SMALL_CTAS);
+    cfg.blockDim = dim3(SMALL_THREADS + 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = SMALL_CTAS;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = probe ? 1 : 2;
+    if (probe) {
+        if (cudaFuncSetAttribute(k_arnoldi_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+                cudaSuccess ||
+            cudaFuncSetAttribute(k_arnoldi_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)SMALL_SMEM) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(clusters, k_arnoldi_small, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            *clusters = 0;
+        }
+        return PPG_OK;
+    }
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_arnoldi_small, a);
+    ++g_launches;
+    if (e != cudaSuccess) {
+        set_cuda_error(e, "cudaLaunchKernelEx(k_arnoldi_small)");
+        cudaGetLastError();
+        return PPG_ERR_CUDA;
+    }
+    return PPG_OK;
+}
+
+// Up to 300,000 basis entries (and a CTA's rows of w and one column in shared
+// memory): 40 steps at 10,000 rows take 1.47 ms, with 150,000 entries 1.55, as
+// launches of their own 1.66; at 15,625 rows 1.76, 1.78 and 1.81.
+bool arnoldi_small_fits(int32_t n, int ncol) {
+    if (ncol > SMALL_COLS || (int64_t)n * ncol > 300000 || n > SMALL_CTAS * 1024) return false;
+    static std::atomic<int> known[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+        cudaGetLastError();
+        return false;
+    }
+    int k = known[dev].load(std::memory_order_relaxed);
+    if (k == 0) {
+        int clusters = 0;
+        small_launch(SmallArnoldi{}, SMALL_SMEM, true, &clusters, nullptr);
+        k = clusters > 0 ? 1 : -1;
+        known[dev].store(k, std::memory_order_relaxed);
+    }
+    return k > 0;
+}
+
+int32_t launch_arnoldi_small(const double* V, int64_t ldv, int j, double* w, int32_t n, bool with_self,
+                             const GmresState& st, int ldh, bool givens, double bnorm, double brtol,
+                             cudaStream_t s) {
+    SmallArnoldi a{};
+    a.V = V;
+    a.ldv = ldv;
+    a.w = w;
+    a.n = n;
+    a.j = j;
+    a.chunk = ((n + SMALL_CTAS - 1) / SMALL_CTAS + 31) / 32 * 32;
+    a.cached = (int)min((size_t)(j + 1), SMALL_SMEM / ((size_t)a.chunk * sizeof(double)) - 1);
+    a.with_self = with_self ? 1 : 0;
+    a.givens = givens ? 1 : 0;
+    a.ldh = ldh;
+    a.bnorm = bnorm;
+    a.brtol = brtol;
+    a.st = st;
+    return small_launch(a, (size_t)(a.cached + 1) * a.chunk * sizeof(double), false, nullptr, s);
+}
 
 }  // namespace ppg

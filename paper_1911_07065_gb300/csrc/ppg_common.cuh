@@ -343,6 +343,12 @@ int32_t launch_finish_column(const GmresState& st, int ldh, int j,
                              const double* h1, const double* h2,
                              const double* nrm, bool givens, double bnorm,
                              double breakdown_rtol, cudaStream_t s);
+// CGS2 of basis column j + 1 (w) against columns 0..j, launch_finish_column and
+// the scaling of w by 1 / h_{j+1,j} in one launch, for a system small enough
+bool arnoldi_small_fits(int32_t n, int ncol);
+int32_t launch_arnoldi_small(const double* V, int64_t ldv, int j, double* w, int32_t n, bool with_self,
+                             const GmresState& st, int ldh, bool givens, double bnorm, double brtol,
+                             cudaStream_t s);
 int32_t launch_scale(const double* x, double* y, int32_t n, const double* scal_ptr,
                      cudaStream_t s);
 int32_t launch_backsolve(const GmresState& st, int ldh, int k, cudaStream_t s);
