@@ -865,7 +865,8 @@ k_spmv_direct(const StepArgs<T> a) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     double sq = 0.0;
     const bool is_long = k1 - k0 > LONG_ROW;
-    if (live && !is_long) {
+    if (live) {
+        if (is_long) k1 = k0;   // (long_rows below)
         const T e0 = a.a0 ? __ldg(a.a0 + r) : T(0);
         const T e1 = (a.a1 && !(a.flags & F_PZERO)) ? a.a1[r] : T(0);
         const T e2 = (a.a2 && (a.flags & F_FINAL)) ? __ldg(a.a2 + r) : T(0);
@@ -881,7 +882,7 @@ k_spmv_direct(const StepArgs<T> a) {
         // loads already brought in)
         for (int32_t k = k0 + PRE; k < k1; ++k)
             acc = fma(__ldg(a.vals + k), __ldg(a.x + __ldg(a.colind + k)), acc);
-        step_epilogue<T, OP>(a, r, acc, e0, e1, e2, sq);
+        if (!is_long) step_epilogue<T, OP>(a, r, acc, e0, e1, e2, sq);
     }
     long_rows<T, OP>(a, r, is_long, sq);
     if constexpr (OP == OP_RESID) {
@@ -1262,16 +1263,14 @@ int32_t launch_step(int op, const StepArgs<T>& a_in, cudaStream_t s) {
         }
         const int most = op == OP_RESID ? 0 : EVEN_MAX;
         // matrix in L2: entries preloaded before the dependency wait.
-        // Up to 5.5 in the average row, FP64: four at 32 registers (2048
-        // threads per SM), five for the plain SpMV step (still 32), five at 40
-        // registers (1536 threads) for the second step of a pair of Algorithm
-        // 1, which spills at 32 (2-D 1000^2 FP64 chains: staged kernel 57.3 ms;
-        // direct with four preloads 55.8 ms (without the evict-last hint 56.3
-        // ms); three for the pair step at 32 registers 55.2 ms; with 128-row
-        // CTAs 54.7 ms; five for the plain SpMV step 53.4 ms; five for the pair
-        // step at 40 registers 52.5 ms, four there 52.8 ms).  FP32: five at 40
-        // registers throughout (40 steps: 400^2 105 -> 94 us, 512^2 137 -> 124
-        // us, 700^2 194 -> 184 us; FP64 700^2 295 -> 298 us).
+        // Up to 5.5 in the average row, five: FP64 at 40 registers (1536 threads
+        // per SM), the plain SpMV step at 32 (2048 threads; it fits), FP32 at 40
+        // (2-D 1000^2 FP64 chains: staged kernel 57.3 ms; direct with four
+        // preloads at 32 registers 55.8 ms, without the evict-last hint 56.3 ms;
+        // with 128-row CTAs 54.7 ms; five for the plain SpMV step 53.4 ms; five
+        // for the pair step at 40 registers 52.5 ms, four there 52.8 ms; 40 steps
+        // of p(A) with four at 32 registers 586 us, five at 40 580 us.  FP32, 40
+        // steps: 400^2 105 -> 94 us, 512^2 137 -> 124 us, 700^2 194 -> 184 us).
         // Above, a seven-entry row whole at 40 registers (FP64 60 x 70 x 80 phi
         // chains of 40 295 -> 268 us, FP32 p chains of 20 100 -> 79 us; 48
         // registers 279 and 80 us, six entries 287 and 88 us), and eight at 64
@@ -1284,12 +1283,10 @@ int32_t launch_step(int op, const StepArgs<T>& a_in, cudaStream_t s) {
             ed = launch_direct<T, 8, 4, true>(cfg, op, a, min(most, 6));   // (above, registers do it)
         else if (a_in.flags & F_WIDE)
             ed = launch_direct<T, 7, 6, true>(cfg, op, a, most);
-        else if (F32 || op == OP_PHI_PAIR2)
-            ed = launch_direct<T, 5, 6, true>(cfg, op, a, most);
-        else if (op == OP_SPMV)
-            ed = launch_direct<T, 5, 8, true>(cfg, op, a, most);
+        else if (!F32 && op == OP_SPMV)
+            ed = launch_even<T, OP_SPMV, 5, 8, true>(cfg, a, most);
         else
-            ed = launch_direct<T, 4, 8, true>(cfg, op, a, most);
+            ed = launch_direct<T, 5, 6, true>(cfg, op, a, most);
         ++g_launches;
         if (ed != cudaSuccess) {
             set_cuda_error(ed, "cudaLaunchKernelEx(k_spmv_direct)");
