@@ -691,7 +691,8 @@ def measure_forms(device, with_oracle=True):
     As = P.A.to_scipy()
     xh32, xh64 = x32.cpu().numpy(), x64.cpu().numpy()
     out["precision_cd3d_160"] = {
-        "p_fp32_roofline": chain_bw(f32t, "p(A) v_j in FP32 (Algorithm 3), every outer step",
+        "p_fp32_roofline": chain_bw(f32t, "p(A) v_j in FP32 (Algorithm 3), every outer step; "
+                                    "in bytes of the CSR, most of which the diagonal form does not read",
                                     "dram_to_algorithmic_p_f32"),
         "phi_fp64_roofline": chain_bw(f64t, "phi(A) v_j in FP64 (Algorithm 1) and p(A) u per restart",
                                       "dram_to_algorithmic_phi_f64"),
