@@ -138,7 +138,7 @@ enum StepFlag : int {
 // row offsets in ascending order.
 constexpr int DIAG_MAX = 32;
 constexpr int DIAG_HEAD = 4 + DIAG_MAX;
-constexpr int DIAG_PAD = 512;   // rows of a diagonal are padded to whole tiles of any step
+constexpr int DIAG_PAD = 1024;  // rows of a diagonal are padded to whole tiles of any step
 struct DiagForm {
     const int32_t* head;   // nullptr: none
     const float* same;     // [DIAG_MAX] the one value of such diagonals

@@ -227,6 +227,12 @@ __host__ __device__ constexpr int step_min_ctas() {
     return sizeof(T) == 4 ? (OP == OP_PHI_PAIR2 ? 6 : 7) : 16;
 }
 
+// ... and of the form that also knows the diagonal steps: 40 registers, for the
+// sake of a matrix without that form, which runs its CSR part (seven random
+// entries per row, 60 steps, 2e6 rows: 2.12 ms with 7 CTAs, 1.89 with 6; the
+// kernel without diagonals 2.05).
+constexpr int DIAG_CTAS = 6;
+
 // one row's multiply-adds over its staged nonzeros [lo, hi): four gathers in
 // flight, then the last 1-3 (FP32: issued together; FP64: one at a time)
 template <typename T, bool WIDE_TAIL>
@@ -283,8 +289,8 @@ __device__ __forceinline__ T row_dot(const T* sval, const int32_t* scol, const T
 // the head and take the CSR path if not, so the host waits for nothing, and
 // the call stays asynchronous and can be captured.
 //
-// 160^3, FP32, 60 steps of p(A): 2.94 -> 1.52 ms (one value per diagonal), 2.93
-// -> 2.15 ms (values of their own), against 49 us a step at 0.91 of the copy
+// 160^3, FP32, 60 steps of p(A): 2.94 -> 1.50 ms (one value per diagonal), 2.93
+// -> 2.28 ms (values of their own), against 49 us a step at 0.91 of the copy
 // bandwidth by CSR.  What is left is the issue of instructions (two thirds of
 // the slots) and the life of a CTA (head, copies, arithmetic: three trips).
 // Tried and slower: reading x and the values straight from global memory (27 -
@@ -294,6 +300,8 @@ __device__ __forceinline__ T row_dot(const T* sval, const int32_t* scol, const T
 // FP64 steps have no use for it: their multiply-adds bound them (504 G FMA/s
 // measured, 1.6 per clock and SM; the chains run at 0.85 - 0.89 of that).
 
+constexpr int DIAG_TILE = step_threads<float>() * step_rpt<float>();   // rows of a tile
+constexpr int DIAG_CAP = 2 * (step_chunk<float>() + 4);   // elements of its shared memory
 constexpr int32_t DIAG_NONE = INT32_MAX;   // no offset: columns are below n
 
 // the head and, behind it, the finder's list
@@ -421,6 +429,7 @@ k_diag_fill(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ coli
         if (used) s_off[rank] = o;
         if (tid == 0) s_same = bad ? 0xffffffffu : bits;
         if (blockIdx.x == 0) {
+            __syncwarp();
             if (used) {
                 H->w[4 + rank] = o;
                 if (one) same[rank] = __int_as_float((int)H->ref[tid]);
@@ -428,6 +437,14 @@ k_diag_fill(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ coli
             if (tid == 0) {
                 H->w[1] = nq;
                 H->w[2] = (int32_t)bits;
+                // two tiles at once where their windows (see diag_tile) fit
+                int at = (nq - __popc(bits)) * 2 * DIAG_TILE, open = 0;
+                for (int q = 0; q < nq; ++q) {
+                    if (q == 0 || s_off[q] - s_off[q - 1] > 16) open = q;
+                    if (q == nq - 1 || s_off[q + 1] - s_off[q] > 16)
+                        at += (2 * DIAG_TILE + (s_off[q] - s_off[open]) + 8 + 3) / 4 * 4;
+                }
+                H->w[3] = at <= DIAG_CAP;
                 if (bad) H->w[0] = 1;
             }
         }
@@ -497,16 +514,20 @@ __device__ __forceinline__ bool diag_arrived(uint32_t bar) {
     return false;
 }
 
-// One tile of a step by diagonals: ROWS rows from row0, NT threads, thread tid
-// on rows tid + i NT.  Warp 0 merges offsets less than 16 apart into windows
+// A tile, or two (halves), of a step by diagonals: ROWS rows from row0, NT
+// threads, thread tid on rows tid + i NT of each half.  Two at once double the
+// bytes in flight and halve what a CTA pays before its copies leave (160^3 p(A)
+// of 60 steps 1.63 -> 1.50 ms, 1500^2 0.81 -> 0.75 ms).  Warp 0 merges offsets less than 16 apart into windows
 // of x, lays windows and values out in the CAP elements of `sm`, and issues
 // the copies: values before the wait on the previous step, windows after it.
 // A tile whose data does not fit (many diagonals with values of their own)
 // reads global memory instead.
 template <typename T, int OP, int NT, int RPT, int CAP>
 __device__ __forceinline__ void diag_tile(const StepArgs<T>& a, int32_t row0, int nrows, float* sm,
-                                          DiagSlot* slot, uint64_t* bar, int* info, double& sq) {
-    constexpr int ROWS = NT * RPT;
+                                          DiagSlot* slot, uint64_t* bar, int* info, double& sq,
+                                          const int halves) {
+    constexpr int HALF = NT * RPT;
+    const int ROWS = HALF * halves;
     const DiagForm& f = a.diag;
     const int tid = threadIdx.x;
     const uint32_t mb = (uint32_t)__cvta_generic_to_shared(bar);
@@ -572,71 +593,83 @@ __device__ __forceinline__ void diag_tile(const StepArgs<T>& a, int32_t row0, in
     } else {
         asm volatile("griddepcontrol.wait;" ::: "memory");
     }
-    T e0[RPT], e1[RPT], e2[RPT], acc[RPT];
+    bool ready = false;
+    for (int h = 0;;) {
+        T e0[RPT], e1[RPT], e2[RPT], acc[RPT];
 #pragma unroll
-    for (int i = 0; i < RPT; ++i) {
-        e0[i] = e1[i] = e2[i] = acc[i] = T(0);
-        const int64_t r = (int64_t)row0 + tid + i * NT;
-        if (tid + i * NT < nrows) {
-            if (a.a0) e0[i] = __ldg(a.a0 + r);
-            if (a.a1 && !(a.flags & F_PZERO)) e1[i] = a.a1[r];
-            if (a.a2 && (a.flags & F_FINAL)) e2[i] = __ldg(a.a2 + r);
-        }
-    }
-    __syncthreads();
-    const bool ready = diag_arrived(mb);
-    if (ready && info[1]) {
-        // rows that lack a diagonal only where a grid ends: most warps have none
-        const unsigned all = 0xffffffffu >> (32 - nq);
-        bool whole = true;
-#pragma unroll
-        for (int i = 0; i < RPT; ++i) whole = whole && b[i] == all;
-        const char* me = reinterpret_cast<const char*>(sm + tid);
-        auto at = [&](int32_t off, int i) {
-            return *reinterpret_cast<const float*>(me + off + i * NT * (int)sizeof(float));
-        };
-        if (__all_sync(0xffffffffu, whole)) {
-#pragma unroll 4
-            for (int q = 0; q < nq; ++q) {
-                const DiagSlot s = slot[q];
-#pragma unroll
-                for (int i = 0; i < RPT; ++i)
-                    acc[i] = fma(s.v == DIAG_SAME ? s.same : at(s.v, i), at(s.x, i), acc[i]);
+        for (int i = 0; i < RPT; ++i) {
+            e0[i] = e1[i] = e2[i] = acc[i] = T(0);
+            const int64_t r = (int64_t)row0 + tid + i * NT;
+            if (tid + i * NT < nrows) {
+                if (a.a0) e0[i] = __ldg(a.a0 + r);
+                if (a.a1 && !(a.flags & F_PZERO)) e1[i] = a.a1[r];
+                if (a.a2 && (a.flags & F_FINAL)) e2[i] = __ldg(a.a2 + r);
             }
-        } else {
-#pragma unroll 4
-            for (int q = 0; q < nq; ++q) {
-                const DiagSlot s = slot[q];
+        }
+        if (h == 0) {
+            __syncthreads();
+            ready = diag_arrived(mb);
+        }
+        if (ready && info[1]) {
+            // rows that lack a diagonal only where a grid ends: most warps have none
+            const unsigned all = 0xffffffffu >> (32 - nq);
+            bool whole = true;
 #pragma unroll
-                for (int i = 0; i < RPT; ++i)
-                    if ((b[i] >> q) & 1)
+            for (int i = 0; i < RPT; ++i) whole = whole && b[i] == all;
+            const char* me = reinterpret_cast<const char*>(sm + tid);
+            auto at = [&](int32_t off, int i) {
+                return *reinterpret_cast<const float*>(me + off + i * NT * (int)sizeof(float));
+            };
+            if (__all_sync(0xffffffffu, whole)) {
+#pragma unroll 4
+                for (int q = 0; q < nq; ++q) {
+                    const DiagSlot s = slot[q];
+#pragma unroll
+                    for (int i = 0; i < RPT; ++i)
                         acc[i] = fma(s.v == DIAG_SAME ? s.same : at(s.v, i), at(s.x, i), acc[i]);
-            }
-        }
-    } else {   // no room, or the copies did not arrive: from global memory
-        for (int q = 0; q < nq; ++q) {
-            const DiagSlot s = slot[q];
-#pragma unroll
-            for (int i = 0; i < RPT; ++i)
-                if ((b[i] >> q) & 1) {
-                    const int64_t r = (int64_t)row0 + tid + i * NT;
-                    acc[i] = fma(s.v == DIAG_SAME ? s.same : __ldg(f.vals + (int64_t)q * f.ld + r),
-                                 __ldg(a.x + r + s.off), acc[i]);
                 }
-        }
-        if (!ready) diag_arrived(mb);   // nothing may land in this CTA's memory after it
-    }
+            } else {
+#pragma unroll 4
+                for (int q = 0; q < nq; ++q) {
+                    const DiagSlot s = slot[q];
 #pragma unroll
-    for (int i = 0; i < RPT; ++i)
-        if (tid + i * NT < nrows)
-            step_epilogue<T, OP>(a, (int64_t)row0 + tid + i * NT, acc[i], e0[i], e1[i], e2[i], sq);
+                    for (int i = 0; i < RPT; ++i)
+                        if ((b[i] >> q) & 1)
+                            acc[i] = fma(s.v == DIAG_SAME ? s.same : at(s.v, i), at(s.x, i), acc[i]);
+                }
+            }
+        } else {   // no room, or the copies did not arrive: from global memory
+            for (int q = 0; q < nq; ++q) {
+                const DiagSlot s = slot[q];
+#pragma unroll
+                for (int i = 0; i < RPT; ++i)
+                    if ((b[i] >> q) & 1) {
+                        const int64_t r = (int64_t)row0 + tid + i * NT;
+                        acc[i] = fma(s.v == DIAG_SAME ? s.same : __ldg(f.vals + (int64_t)q * f.ld + r),
+                                     __ldg(a.x + r + s.off), acc[i]);
+                    }
+            }
+            if (!ready) diag_arrived(mb);   // nothing may land in this CTA's memory after it
+        }
+#pragma unroll
+        for (int i = 0; i < RPT; ++i)
+            if (tid + i * NT < nrows)
+                step_epilogue<T, OP>(a, (int64_t)row0 + tid + i * NT, acc[i], e0[i], e1[i], e2[i], sq);
+        if (++h == halves) break;
+        row0 += HALF;
+        nrows -= HALF;
+        sm += HALF;
+#pragma unroll
+        for (int i = 0; i < RPT; ++i)
+            b[i] = tid + i * NT < nrows ? diag_bits(f, row0 + tid + i * NT) : 0;
+    }
 }
 
 // PF: prefetch the tile a.pf_ahead tiles ahead (half a resident wave) into
 // L2 (launched when the matrix is not held in an L2 set-aside)
 // DG: the (FP32) matrix is at hand by its diagonals too, if it has that form
 template <typename T, int OP, bool PF, bool DG>
-__global__ void __launch_bounds__(step_threads<T>(), step_min_ctas<T, OP>())
+__global__ void __launch_bounds__(step_threads<T>(), DG ? DIAG_CTAS : step_min_ctas<T, OP>())
 k_spmv_step(const StepArgs<T> a) {
     constexpr int NT = step_threads<T>();      // threads per CTA
     // staging copies start at a chunk base rounded down to 4 elements
@@ -667,8 +700,14 @@ k_spmv_step(const StepArgs<T> a) {
             __shared__ uint64_t bar;
             __shared__ int info[2];
             double sq = 0.0;
-            diag_tile<T, OP, NT, RPT, (CHUNK + PAD) * 2>(a, (int32_t)row0, nrows, (float*)stage, slot,
-                                                        &bar, info, sq);
+            int halves = 1, rows = nrows;
+            if (OP != OP_RESID && __ldg(a.diag.head + 3)) {   // two tiles on every other CTA
+                if (blockIdx.x & 1) return;
+                halves = (int64_t)a.n - row0 > ROWS ? 2 : 1;
+                rows = (int)min((int64_t)a.n - row0, (int64_t)2 * ROWS);
+            }
+            diag_tile<T, OP, NT, RPT, DIAG_CAP>(a, (int32_t)row0, rows, (float*)stage, slot, &bar, info,
+                                                sq, halves);
             if constexpr (OP == OP_RESID) block_sq<NT>(sq, sred, a.part);
             return;
         }
@@ -1103,22 +1142,19 @@ static int step_resident_ctas() {
 // repay building it: about two passes over the matrix, 60 us for 1e6 rows of
 // five entries and 160 us for 4.1e6 rows of seven.  Per step, CSR against
 // diagonals (one value per diagonal / values of their own):
-//   streamed from HBM, 160^3:     49 us   24.4 us / 34 us   (repaid by 14 steps)
-//   held in L2, 1001 x 997:       9.0 us   6.2 us / 7.0 us  (repaid by 30)
-//   held in L2, 301 x 299:        2.2 us   -      / 2.3 us
-// (a matrix held in L2 is bound by what its CTAs of 128 rows cost to launch,
-// about 1 ns each, which smaller matrices do not feel).
-constexpr int64_t DIAG_MIN_STEPS = 20, DIAG_MIN_STEPS_L2 = 32;
-constexpr int32_t DIAG_MIN_ROWS_L2 = 700000;
+//   160^3:     49 us   24.2 us / 37 us   (repaid by 14 steps)
+// A matrix held in L2 stays with the direct steps: by diagonals a grid would gain
+// (1000^2, 60 steps: 0.53 -> 0.38 ms), but whether it is one is known on the device
+// alone, and a matrix that is not would lose more than the direct steps' gain
+// (1.2e6 rows of seven random entries, 60 steps: 0.76 -> 1.07 ms).
+constexpr int64_t DIAG_MIN_STEPS = 20;
 
 int32_t DiagStore::build(const int32_t* rowptr, const int32_t* colind, const float* vals, int32_t n,
                          int64_t nnz, int64_t steps, cudaStream_t stream) {
     if (n <= DIRECT_MAX_N || n > (1 << 30) || steps < DIAG_MIN_STEPS || nnz < n) return PPG_OK;
     const int dev = current_device();
     if (dev < 0) return PPG_OK;
-    if (fits_l2(8.0 * nnz + 16.0 * n, l2_bytes(dev)) &&
-        (n < DIAG_MIN_ROWS_L2 || steps < DIAG_MIN_STEPS_L2))
-        return PPG_OK;
+    if (fits_l2(8.0 * nnz + 16.0 * n, l2_bytes(dev))) return PPG_OK;
     const double avg = (double)nnz / (double)n;
     const int most = (int)std::min<double>(DIAG_MAX, 2.0 * avg + 0.5);
     if (avg > most) return PPG_OK;

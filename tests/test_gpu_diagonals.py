@@ -1,7 +1,7 @@
 """GPU: FP32 chains by diagonals against the CSR steps, bit for bit.
 
-ppg_apply_poly builds the diagonal form of a matrix for long FP32 chains;
-ppg_apply_poly_noalloc, which has no memory for it, always runs the CSR steps.
+ppg_apply_poly builds the diagonal form of a matrix for long FP32 chains.  The
+same rows at the head of a matrix with many offsets take the CSR steps.
 """
 import numpy as np
 import pytest
@@ -11,7 +11,7 @@ from gpu_util import dev_csr, ppg_or_skip, to_dev
 
 pytestmark = pytest.mark.gpu
 
-N = 720_003   # not a multiple of any tile; held in L2, large enough for the form
+N = 2_600_003   # not a multiple of any tile; larger than L2; an odd number of tiles
 
 
 @pytest.fixture(scope="module")
@@ -19,13 +19,13 @@ def env():
     return ppg_or_skip()
 
 
-def _banded(offsets, one_value=(), drop=0.0, empty=(), seed=0):
-    """Rows of N with entries at `offsets` (inside the matrix), each left out
+def _banded(offsets, one_value=(), drop=0.0, empty=(), seed=0, n=N):
+    """n rows with entries at `offsets` (inside the matrix), each left out
     with probability `drop`; diagonals in `one_value` have a single value."""
     rng = np.random.default_rng(seed)
     off = np.array(sorted(offsets), dtype=np.int64)
-    cols = np.arange(N)[:, None] + off[None, :]
-    valid = (cols >= 0) & (cols < N)
+    cols = np.arange(n)[:, None] + off[None, :]
+    valid = (cols >= 0) & (cols < n)
     if drop:
         valid &= (rng.random(cols.shape) >= drop) | (off[None, :] == 0)
     valid[list(empty)] = False
@@ -34,10 +34,18 @@ def _banded(offsets, one_value=(), drop=0.0, empty=(), seed=0):
         if o in one_value:
             vals[:, i] = -0.75 / off.size
         if o == 0:
-            vals[:, i] = 4.0 if 0 in one_value else 4.0 + 0.1 * rng.random(N)
-    rowptr = np.zeros(N + 1, dtype=np.int64)
+            vals[:, i] = 4.0 if 0 in one_value else 4.0 + 0.1 * rng.random(n)
+    rowptr = np.zeros(n + 1, dtype=np.int64)
     rowptr[1:] = np.cumsum(valid.sum(1))
-    return synth.CSRHost(N, rowptr.astype(np.int32), cols[valid].astype(np.int32), vals[valid])
+    return synth.CSRHost(n, rowptr.astype(np.int32), cols[valid].astype(np.int32), vals[valid])
+
+
+def _csr_steps(p, torch, A, R, v):
+    """p(A) v by the CSR steps: 100 rows more, each with an offset of its own."""
+    k = torch.arange(100, dtype=torch.int32, device="cuda")
+    big = p.CSR(torch.cat([A.rowptr, A.nnz + 1 + k]), torch.cat([A.colind, A.n - 99 * k]),
+                torch.cat([A.vals, torch.ones(100, dtype=torch.float32, device="cuda")]))
+    return p.apply_poly(big, R, torch.cat([v, v[:100]]))[: A.n]
 
 
 def _roots():
@@ -54,6 +62,7 @@ def _roots():
 GRID = (-887, -1, 0, 1, 887)
 CASES = {
     "one_value_each": dict(offsets=GRID, one_value=GRID),
+    "an_even_number_of_tiles": dict(offsets=GRID, one_value=GRID, n=N + 512),
     "some_own_values": dict(offsets=GRID, one_value=(-887, 0, 887)),
     "dropped_entries": dict(offsets=GRID, drop=0.3, empty=(0, 511, 512, N - 1)),
     "close_offsets": dict(offsets=(-17, -16, -2, 0, 3, 18, 19)),
@@ -72,10 +81,10 @@ def test_diagonals_equal_csr_steps(env, name, shift):
     A = dev_csr(p, torch, _banded(**CASES[name]), dtype=torch.float32)
     R = p.Roots.from_complex(_roots())
     # shift: v and y off a 16-byte boundary
-    buf = to_dev(torch, np.random.default_rng(5).standard_normal(N + 4), torch.float32)
-    v = buf[shift:shift + N]
-    y = torch.empty(N + 4, dtype=torch.float32, device="cuda")[shift:shift + N]
-    ref = p.apply_poly_noalloc(A, R, v, torch.empty_like(v))
+    buf = to_dev(torch, np.random.default_rng(5).standard_normal(A.n + 4), torch.float32)
+    v = buf[shift:shift + A.n]
+    y = torch.empty(A.n + 4, dtype=torch.float32, device="cuda")[shift:shift + A.n]
+    ref = _csr_steps(p, torch, A, R, v)
     p.apply_poly(A, R, v, out=y)
     torch.cuda.synchronize()
     assert torch.isfinite(ref).all()
@@ -90,7 +99,7 @@ def test_unsorted_row_keeps_the_csr_steps(env):
     A = p.CSR.from_host(H.rowptr, H.colind, H.vals, dtype=torch.float32, validate=False)
     R = p.Roots.from_complex(_roots())
     v = to_dev(torch, np.random.default_rng(6).standard_normal(N), torch.float32)
-    ref = p.apply_poly_noalloc(A, R, v, torch.empty_like(v))
+    ref = _csr_steps(p, torch, A, R, v)
     assert torch.equal(p.apply_poly(A, R, v), ref)
 
 
@@ -117,7 +126,7 @@ def test_values_seen_by_the_next_call(env):
     p.apply_poly(A, R, v)
     A.vals[A.nnz // 2] += 0.25
     A.vals[7] = float("inf")
-    ref = p.apply_poly_noalloc(A, R, v, torch.empty_like(v))
+    ref = _csr_steps(p, torch, A, R, v)
     got = p.apply_poly(A, R, v)
     assert torch.equal(torch.nan_to_num(got), torch.nan_to_num(ref))
     assert torch.equal(torch.isfinite(got), torch.isfinite(ref))
