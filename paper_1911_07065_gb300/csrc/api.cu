@@ -143,14 +143,17 @@ static int32_t run_steps(const std::vector<Step>& plan, int i0, int i1, const in
         if (bytes_out) *bytes_out = 0.0;
         return PPG_OK;
     }
+    // (a small system reserves its share of L2 too, though its one launch makes no
+    // use of it: a larger one may come next inside a stream capture, where the
+    // limit cannot change)
+    int32_t keep_rows = 0;
+    const int keep = keep_a_flag(n, nnz, (int)sizeof(T), 3, reserve_l2, &keep_rows);
     if (i0 == 0 && i1 == (int)plan.size() && chain_cluster_fits<T>(plan, n, nnz)) {
         PPG_TRY(launch_chain_cluster<T>(plan, rowptr, colind, vals, n, bufs, s));
         for (const Step& st : plan) bytes += step_bytes(st.op, st.flags, n, nnz, (int)sizeof(T));
         if (bytes_out) *bytes_out = bytes;
         return PPG_OK;
     }
-    int32_t keep_rows = 0;
-    const int keep = keep_a_flag(n, nnz, (int)sizeof(T), 3, reserve_l2, &keep_rows);
     const int sms = device_sm_count();
     for (int i = i0; i < i1; ++i) {
         const Step& st = plan[(size_t)i];

@@ -1,5 +1,9 @@
 """GPU: a small system's chain in one launch against the step-by-step chain,
 bit for bit."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -73,3 +77,28 @@ def test_one_launch_inside_a_graph_and_on_two_streams(env):
             outs.append(p.apply_poly(A, R, v))
     torch.cuda.synchronize()
     assert torch.equal(y, ref) and all(torch.equal(o, ref) for o in outs)
+
+
+def test_capture_of_a_larger_system_after_a_small_one(env):
+    """In a fresh process: the small system's call leaves the L2 share that the
+    larger one's chain needs, which could not be set inside a capture."""
+    code = """
+import numpy as np, torch, synth, paper_1911_07065_gb300 as p
+R = p.Roots.from_complex(np.array([5 + 2j, 5 - 2j] * 15))
+def system(n):
+    H = synth.cd2d(n, 0.5)
+    A = p.CSR.from_host(H.rowptr, H.colind, H.vals, device="cuda")
+    return A, torch.ones(A.n, dtype=torch.float64, device="cuda")
+A, v = system(50)
+p.apply_poly(A, R, v)
+A, v = system(150)
+y = torch.empty_like(v)
+torch.cuda.synchronize()
+g = torch.cuda.CUDAGraph()
+with torch.cuda.graph(g, stream=torch.cuda.Stream()):
+    p.apply_poly(A, R, v, out=y)
+g.replay()
+assert torch.equal(y, p.apply_poly(A, R, v))
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=root, timeout=120)
