@@ -233,6 +233,16 @@ int32_t ppg_apply_poly_noalloc(const ppg_csr* A, const ppg_roots* r,
 int32_t ppg_apply_phi(const ppg_csr* A, const ppg_roots* r, const void* v,
                       void* y, void* stream);
 
+/* How ppg_apply_poly and ppg_apply_phi would run a chain of `steps` root steps
+ * over A, for callers that look into a run time: one of PPG_FORM_*.
+ * Synchronises. */
+#define PPG_FORM_STAGED      0   /* a launch per step, entries staged from memory */
+#define PPG_FORM_DIRECT      1   /* a launch per step, entries read in place (small, or in L2) */
+#define PPG_FORM_CLUSTER     2   /* the whole chain in one launch of one thread-block cluster */
+#define PPG_FORM_DIAGONALS   3   /* a launch per step, FP32 matrix by its diagonals */
+#define PPG_FORM_DIAGONALS_2 4   /* the same, two tiles per thread block */
+int32_t ppg_chain_form(const ppg_csr* A, int32_t steps, int32_t* form, void* stream);
+
 /* y = A x.  Asynchronous. */
 int32_t ppg_spmv(const ppg_csr* A, const void* x, void* y, void* stream);
 

@@ -116,6 +116,7 @@ def _load():
         "ppg_apply_phi": (c_i32, [C.POINTER(ppg_csr), C.POINTER(ppg_roots), c_vp, c_vp, c_vp]),
         "ppg_apply_poly_noalloc": (c_i32, [C.POINTER(ppg_csr), C.POINTER(ppg_roots), c_vp,
                                            c_vp, c_vp]),
+        "ppg_chain_form": (c_i32, [C.POINTER(ppg_csr), c_i32, C.POINTER(c_i32), c_vp]),
         "ppg_spmv": (c_i32, [C.POINTER(ppg_csr), c_vp, c_vp, c_vp]),
         "ppg_solve": (c_i32, [C.POINTER(ppg_csr), C.POINTER(ppg_roots), c_vp, c_vp, c_i32,
                               c_f64, C.POINTER(ppg_opts), C.POINTER(ppg_stats), c_vp]),
@@ -154,7 +155,7 @@ EXPORTS = (
     "ppg_launch_count",
     "ppg_harmonic_ritz", "ppg_leja_order", "ppg_add_roots", "ppg_roots_from_hessenberg",
     "ppg_csr_validate_host", "ppg_build_poly", "ppg_apply_poly", "ppg_apply_phi",
-    "ppg_spmv", "ppg_solve", "ppg_solve_flex", "ppg_stability_check",
+    "ppg_chain_form", "ppg_spmv", "ppg_solve", "ppg_solve_flex", "ppg_stability_check",
     "ppg_csr_transpose", "ppg_adjoint_vals_grad", "ppg_apply_poly_noalloc",
     "ppg_solve_batched", "ppg_build_poly_composite", "ppg_solve_double", "ppg_solve_chpoly",
     "ppg_build_poly_checked", "ppg_sweep_plan_create", "ppg_sweep_plan_info",

@@ -156,6 +156,17 @@ def apply_phi(A: CSR, roots: Roots, v: torch.Tensor, out: Optional[torch.Tensor]
     return y
 
 
+CHAIN_FORMS = ("staged", "direct", "cluster", "diagonals", "diagonals_2")
+
+
+def chain_form(A: CSR, steps: int, stream=None) -> str:
+    """How apply_poly and apply_phi run a chain of ``steps`` root steps over A
+    (one of CHAIN_FORMS)."""
+    form = C.c_int32()
+    check(lib.ppg_chain_form(A.ref(), steps, C.byref(form), _stream(stream)), "ppg_chain_form")
+    return CHAIN_FORMS[form.value]
+
+
 def spmv(A: CSR, x: torch.Tensor, out: Optional[torch.Tensor] = None, stream=None):
     _need_cuda(x)
     y = torch.empty_like(x) if out is None else out

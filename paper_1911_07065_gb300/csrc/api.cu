@@ -148,7 +148,7 @@ static int32_t run_steps(const std::vector<Step>& plan, int i0, int i1, const in
     // limit cannot change)
     int32_t keep_rows = 0;
     const int keep = keep_a_flag(n, nnz, (int)sizeof(T), 3, reserve_l2, &keep_rows);
-    if (i0 == 0 && i1 == (int)plan.size() && chain_cluster_fits<T>(plan, n, nnz)) {
+    if (i0 == 0 && i1 == (int)plan.size() && chain_cluster_fits<T>(plan.size(), n, nnz)) {
         PPG_TRY(launch_chain_cluster<T>(plan, rowptr, colind, vals, n, bufs, s));
         for (const Step& st : plan) bytes += step_bytes(st.op, st.flags, n, nnz, (int)sizeof(T));
         if (bytes_out) *bytes_out = bytes;
@@ -616,8 +616,8 @@ static int32_t run_solve(SolveCore& c) {
     // (a chain that is one launch goes ahead whole: its result, basis column
     // j + 2, is not read by the update either)
     const bool whole = chain && !c.sweep &&
-                       (c.flex ? chain_cluster_fits<float>(*chain, n, nnz)
-                               : chain_cluster_fits<double>(*chain, n, nnz));
+                       (c.flex ? chain_cluster_fits<float>(chain->size(), n, nnz)
+                               : chain_cluster_fits<double>(chain->size(), n, nnz));
     const int nahead = whole ? (int)chain->size()
                        : (chain && !c.sweep)
                            ? std::max(0, std::min(kLookahead, (int)chain->size() - 1))
@@ -1205,6 +1205,35 @@ int32_t ppg_apply_poly(const ppg_csr* A, const ppg_roots* r, const void* v, void
 int32_t ppg_apply_phi(const ppg_csr* A, const ppg_roots* r, const void* v, void* y,
                       void* stream) {
     return apply_common(A, r, v, y, stream, true);
+}
+
+int32_t ppg_chain_form(const ppg_csr* A, int32_t steps, int32_t* form, void* stream) {
+    PPG_TRY(check_csr(A, -1));
+    if (!form || steps < 1) return PPG_ERR_ARG;
+    PPG_TRY(setup_device_pool());
+    cudaStream_t s = (cudaStream_t)stream;
+    const bool f64 = A->dtype == PPG_F64;
+    if (f64 ? chain_cluster_fits<double>((size_t)steps, A->n, A->nnz)
+            : chain_cluster_fits<float>((size_t)steps, A->n, A->nnz)) {
+        *form = PPG_FORM_CLUSTER;
+        return PPG_OK;
+    }
+    if (!f64) {
+        DiagStore diag;
+        PPG_TRY(diag.build(A->rowptr, A->colind, (const float*)A->vals, A->n, A->nnz, steps, s));
+        if (diag.f.head) {
+            int32_t head[4] = {1, 0, 0, 0};
+            PPG_CUDA(cudaMemcpyAsync(head, diag.f.head, sizeof(head), cudaMemcpyDeviceToHost, s));
+            PPG_CUDA(cudaStreamSynchronize(s));
+            if (head[0] == 0) {
+                *form = head[3] ? PPG_FORM_DIAGONALS_2 : PPG_FORM_DIAGONALS;
+                return PPG_OK;
+            }
+        }
+    }
+    const bool direct = A->n <= DIRECT_MAX_N || (keep_a_flag(A->n, A->nnz, f64 ? 8 : 4, 3) & F_KEEP_A);
+    *form = direct ? PPG_FORM_DIRECT : PPG_FORM_STAGED;
+    return PPG_OK;
 }
 
 int32_t ppg_build_poly(const ppg_csr* A, int32_t d, const double* v0, const ppg_opts* opts,

@@ -262,9 +262,9 @@ int32_t run_plan(const std::vector<Step>& plan, const int32_t* rowptr,
                  bool reserve_l2 = true, DiagStore* diag = nullptr);
 
 // A small system's whole chain in one launch (small_chain.cu): whether it takes
-// the plan, and the plan's steps with the same buffers as run_plan's.
+// a plan of `steps` steps, and the plan's steps with the same buffers as run_plan's.
 template <typename T>
-bool chain_cluster_fits(const std::vector<Step>& plan, int32_t n, int64_t nnz);
+bool chain_cluster_fits(size_t steps, int32_t n, int64_t nnz);
 template <typename T>
 int32_t launch_chain_cluster(const std::vector<Step>& plan, const int32_t* rowptr,
                              const int32_t* colind, const T* vals, int32_t n, const Buffers& bufs,

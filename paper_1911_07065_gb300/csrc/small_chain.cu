@@ -279,14 +279,14 @@ bool cluster_possible() {
 // 100^2 86 / 79 us, 110^2 85 / 90 us; 3-D 20^3 86 / 79 us, 25^3 85 / 133 us), FP32
 // up to two rows a thread (50^2 83 / 21 us, 128^2 84 / 36 us).
 template <typename T>
-bool chain_cluster_fits(const std::vector<Step>& plan, int32_t n, int64_t nnz) {
+bool chain_cluster_fits(size_t steps, int32_t n, int64_t nnz) {
     if (n > CHAIN_CTAS * CHAIN_THREADS * CHAIN_ROWS) return false;
     if (nnz + n > (sizeof(T) == 8 ? 64000 : 200000)) return false;
-    if (plan.size() < 2 || plan.size() > (size_t)CHAIN_STEPS) return false;
+    if (steps < 2 || steps > (size_t)CHAIN_STEPS) return false;
     return cluster_possible<T>();
 }
-template bool chain_cluster_fits<double>(const std::vector<Step>&, int32_t, int64_t);
-template bool chain_cluster_fits<float>(const std::vector<Step>&, int32_t, int64_t);
+template bool chain_cluster_fits<double>(size_t, int32_t, int64_t);
+template bool chain_cluster_fits<float>(size_t, int32_t, int64_t);
 
 template <typename T>
 int32_t launch_chain_cluster(const std::vector<Step>& plan, const int32_t* rowptr,
