@@ -313,109 +313,219 @@ struct DiagHead {
 };
 constexpr uint32_t DIAG_UNSET = 0x7fb4deadu;   // a NaN that no arithmetic returns
 
-__global__ void k_diag_init(DiagHead* H) {
+// The list starts with the middle row's offsets (of a grid, all of them), so that
+// the CTAs of k_diag_find, which end together, have little to add to it.
+__global__ void k_diag_init(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colind,
+                            const float* __restrict__ vals, int32_t n, int32_t most, DiagHead* H) {
     const int i = threadIdx.x;
-    if (i < DIAG_HEAD) H->w[i] = 0;
+    const int32_t r = n / 2, k = __ldg(rowptr + r), len = __ldg(rowptr + r + 1) - k;
+    if (i < DIAG_HEAD) H->w[i] = i == 0 && len > most ? 1 : 0;
     if (i < DIAG_MAX) {
-        H->off[i] = DIAG_NONE;
-        H->ref[i] = DIAG_UNSET;
+        const bool has = i < len && len <= most;
+        // (not increasing: k_diag_find sees it; no offset is in the list twice)
+        const int32_t o = has ? __ldg(colind + k + i) - r : DIAG_NONE;
+        const bool first = i == 0 || !has || o > __ldg(colind + k + i - 1) - r;
+        H->off[i] = first ? o : DIAG_NONE;
+        H->ref[i] = has && first ? __float_as_uint(__ldg(vals + k + i)) : DIAG_UNSET;
     }
     if (i == 0) H->mixed = 0;
 }
 
 // Every offset of the matrix into the list, and whether its values are all the
-// same.  A CTA takes DIAG_ROWS rows: each round it finds the rows' smallest
-// next offset, the rows that hold it and whether their values agree; at the
-// end one warp compares its findings with the list and adds what is new.
+// same.  A CTA takes tiles of DIAG_ROWS rows in turn, copies their entries to
+// shared memory (coalesced) and walks them there, one row per thread, beside its
+// own sorted list of the offsets so far; what the list lacks is merged into it and
+// the tile walked again, which for a grid happens once or twice in all.  At the
+// end one warp compares that list with the matrix's and adds what is new.
 constexpr int DIAG_ROWS = 128;
-__global__ void __launch_bounds__(DIAG_ROWS)
+constexpr int DIAG_STAGE = 2048;   // entries in shared memory at once
+__device__ __forceinline__ int diag_at(int i) { return i + (i >> 5); }   // (no bank conflicts)
+
+__global__ void __launch_bounds__(DIAG_ROWS, 10)
 k_diag_find(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colind,
             const float* __restrict__ vals, int32_t n, int32_t most, DiagHead* H) {
-    constexpr int NW = DIAG_ROWS / 32;
-    __shared__ int32_t s_min[2][NW];
-    __shared__ int32_t s_off[DIAG_MAX];
-    __shared__ uint32_t s_ref[DIAG_MAX];
-    __shared__ int s_bad;
+    __shared__ int32_t s_col[DIAG_STAGE + DIAG_STAGE / 32];
+    __shared__ int32_t s_val[DIAG_STAGE + DIAG_STAGE / 32];   // (bits)
+    __shared__ int2 s_list[DIAG_MAX + 1];                     // offset, bits of its first value
+    __shared__ int2 s_new[DIAG_MAX];
+    __shared__ int s_to[DIAG_MAX];                            // where the list's entries went
+    __shared__ int32_t s_first, s_end, s_bad, s_longest;
+    __shared__ uint32_t s_mixed;
     const int tid = threadIdx.x, lane = tid & 31;
-    if (tid == 0) s_bad = *(volatile int32_t*)&H->w[0];
-    __syncthreads();
-    if (s_bad) return;   // another CTA has seen that there is no such form
-    const int64_t r = (int64_t)blockIdx.x * DIAG_ROWS + tid;
-    int32_t k = 0, e = 0;
-    if (r < n) {
-        k = __ldg(rowptr + r);
-        e = __ldg(rowptr + r + 1);
+    if (tid <= DIAG_MAX) s_list[tid].x = DIAG_NONE;
+    if (tid == 0) {
+        s_mixed = 0;
+        s_longest = 0;
     }
-    int32_t cur = k < e ? __ldg(colind + k) - (int32_t)r : DIAG_NONE;
+    uint32_t mixed = 0;   // bit q: entry q of the list has several values, by this thread's rows
     bool ok = true;
-    unsigned mixed = 0;
-    int q = 0;
-    for (;; ++q) {
-        const int32_t wm = __reduce_min_sync(0xffffffffu, cur);
-        if (lane == 0) s_min[q & 1][tid >> 5] = wm;
-        __syncthreads();
-        int32_t m = s_min[q & 1][0];
-#pragma unroll
-        for (int w = 1; w < NW; ++w) m = min(m, s_min[q & 1][w]);
-        if (m == DIAG_NONE || q == most) {   // uniform
-            ok = ok && m == DIAG_NONE;
-            break;
+    // the next tile's row, and whether another CTA has seen that there is no such
+    // form, are read a tile ahead
+    const int32_t step = gridDim.x * DIAG_ROWS;   // (n and step: below 2^31 together)
+    int32_t row0 = blockIdx.x * DIAG_ROWS, next_k = 0, next_e = 0, next_bad = 0;
+    auto ahead = [&](int32_t row) {
+        if (row + tid < n) {
+            next_k = __ldg(rowptr + row + tid);
+            next_e = __ldg(rowptr + row + tid + 1);
         }
-        const bool hit = cur == m;
-        uint32_t v = 0;
-        if (hit) {
-            v = __float_as_uint(__ldg(vals + k));
-            s_ref[q] = v;   // any of them
-            s_off[q] = m;
-            ++k;
-            cur = k < e ? __ldg(colind + k) - (int32_t)r : DIAG_NONE;
-            ok = ok && cur > m;   // columns increase within the row
+        if (tid == 0) next_bad = *(volatile int32_t*)&H->w[0];
+    };
+    ahead(row0);
+    for (; row0 < n; row0 += step) {
+        const int32_t r = row0 + tid;
+        const bool opening = row0 == (int32_t)blockIdx.x * DIAG_ROWS;
+        int32_t k = 0, e = 0;
+        if (tid == 0) s_bad = next_bad;
+        if (r < n) {
+            k = next_k;
+            e = next_e;
+            ok = ok && e - k <= most;
+            if (tid == 0) s_first = k;
+            if (tid == DIAG_ROWS - 1 || r == n - 1) s_end = e;
         }
-        __syncthreads();
-        if (!__syncthreads_and(!hit || v == s_ref[q])) mixed |= 1u << q;
+        ahead(row0 + step);
+        if (__syncthreads_or(!ok)) break;
+        if (s_bad) return;
+        const int32_t first = s_first, end = s_end;
+        if (opening) {   // the list to start with: the longest row's
+            atomicMax(&s_longest, (e - k) << 7 | tid);
+            __syncthreads();
+            const int len = s_longest >> 7;
+            if (tid < len) {
+                const int32_t rr = row0 + (s_longest & 127), kk = __ldg(rowptr + rr) + tid;
+                s_list[tid] = {__ldg(colind + kk) - rr, __float_as_int(__ldg(vals + kk))};
+            }
+        }
+        for (;;) {
+            int32_t before = INT32_MIN, miss = DIAG_NONE, miss_v = 0;
+            int q = 0;
+            int32_t kk = k;
+            __syncthreads();
+            for (int32_t c0 = first, c1; c0 < end; c0 = c1) {
+                c1 = c0 + min(end - c0, DIAG_STAGE);
+#pragma unroll 4
+                for (int32_t i = tid; i < c1 - c0; i += DIAG_ROWS) {
+                    s_col[diag_at(i)] = __ldg(colind + c0 + i);
+                    s_val[diag_at(i)] = __float_as_int(__ldg(vals + c0 + i));
+                }
+                __syncthreads();
+                const int32_t stop = min(e, c1);
+                for (; kk < stop; ++kk) {
+                    const int i = diag_at(kk - c0);
+                    const int32_t o = s_col[i] - r;
+                    if (o <= before) {   // columns increase within the row
+                        ok = false;
+                        kk = e;
+                        break;
+                    }
+                    before = o;
+                    int2 w = s_list[q];
+                    while (w.x < o) w = s_list[++q];   // (ends at DIAG_NONE)
+                    if (w.x == o) {
+                        if (w.y != s_val[i]) mixed |= 1u << q;
+                    } else if (miss == DIAG_NONE) {
+                        miss = o;
+                        miss_v = s_val[i];
+                    }
+                }
+                __syncthreads();
+            }
+            if (!__syncthreads_or(miss != DIAG_NONE || !ok)) break;
+            if (tid < DIAG_MAX) s_new[tid].x = DIAG_NONE;
+            __syncthreads();
+            if (miss != DIAG_NONE) {
+                int slot = 0;
+                for (; slot < DIAG_MAX; ++slot) {
+                    const int32_t old = atomicCAS(&s_new[slot].x, DIAG_NONE, miss);
+                    if (old == DIAG_NONE || old == miss) break;
+                }
+                if (slot < DIAG_MAX) s_new[slot].y = miss_v;   // any of them
+                ok = ok && slot < DIAG_MAX;
+            }
+            __syncthreads();
+            if (tid < 32) {
+                const int2 a = s_list[lane], b = s_new[lane];
+                int to_a = lane, to_b = 0;
+                for (int i = 0; i < 32; ++i) {
+                    const int32_t ai = __shfl_sync(0xffffffffu, a.x, i), bi = __shfl_sync(0xffffffffu, b.x, i);
+                    to_a += bi < a.x;
+                    to_b += (ai < b.x) + (bi < b.x);
+                }
+                ok = ok && !(b.x != DIAG_NONE && to_b >= most) && !(a.x != DIAG_NONE && to_a >= most);
+                if (__all_sync(0xffffffffu, ok)) {   // (most <= DIAG_MAX)
+                    if (a.x != DIAG_NONE) s_list[to_a] = a;
+                    if (b.x != DIAG_NONE) s_list[to_b] = b;
+                    s_to[lane] = to_a;
+                }
+            }
+            if (__syncthreads_or(!ok)) break;
+            uint32_t was = mixed;
+            for (mixed = 0; was; was &= was - 1) mixed |= 1u << s_to[__ffs(was) - 1];
+        }
     }
-    ok = __syncthreads_and(ok);
-    if (!ok) {
+    static_assert(DIAG_MAX == 32, "a bit, and a lane, for each");
+    mixed = __reduce_or_sync(0xffffffffu, mixed);
+    if (lane == 0) atomicOr(&s_mixed, mixed);
+    if (__syncthreads_or(!ok)) {
         if (tid == 0) atomicExch(&H->w[0], 1);
         return;
     }
     if (tid >= 32) return;
-    // lane i < q: this CTA's offset i against the list (one load), then
-    // whatever the list does not have yet
+    // lane i: this CTA's offset i against the list (one load), then whatever the
+    // list does not have yet
     const int32_t have = *(volatile int32_t*)&H->off[lane];
-    const unsigned gmixed = *(volatile uint32_t*)&H->mixed;
-    const int32_t mine = lane < q ? s_off[lane] : DIAG_NONE;
+    const uint32_t gmixed = *(volatile uint32_t*)&H->mixed;
+    const int32_t mine = s_list[lane].x;
     int slot = -1;
     for (int i = 0; i < DIAG_MAX; ++i)
         if (__shfl_sync(0xffffffffu, have, i) == mine && mine != DIAG_NONE) slot = i;
     if (mine != DIAG_NONE && slot < 0)
         for (int i = 0; i < DIAG_MAX && slot < 0; ++i) {
-            const int32_t old = atomicCAS(&H->off[i], DIAG_NONE, mine);
+            int32_t old = *(volatile int32_t*)&H->off[i];
+            if (old == DIAG_NONE) old = atomicCAS(&H->off[i], DIAG_NONE, mine);
             if (old == DIAG_NONE || old == mine) slot = i;
         }
+    uint32_t add = 0;
     if (mine != DIAG_NONE) {
         if (slot < 0) {
             atomicExch(&H->w[0], 1);
         } else if (!((gmixed >> slot) & 1)) {
-            const uint32_t v = s_ref[lane];
+            const uint32_t v = (uint32_t)s_list[lane].y;
             uint32_t ref = *(volatile uint32_t*)&H->ref[slot];
             if (ref == DIAG_UNSET) {
                 ref = atomicCAS(&H->ref[slot], DIAG_UNSET, v);
                 if (ref == DIAG_UNSET) ref = v;
             }
-            if (((mixed >> lane) & 1) || ref != v || v == DIAG_UNSET)
-                atomicOr(&H->mixed, 1u << slot);
+            if (((s_mixed >> lane) & 1) || ref != v || v == DIAG_UNSET) add = 1u << slot;
         }
     }
+    add = __reduce_or_sync(0xffffffffu, add);
+    if (lane == 0 && add) atomicOr(&H->mixed, add);
 }
 
-// the form itself, one row per thread, from the finished list
+// elements of shared memory that `rows` rows of a matrix with nq offsets, `owns` of
+// them with values of their own, take in diag_tile
+__device__ __forceinline__ int diag_room(const int32_t* off, int nq, int owns, int rows) {
+    int at = owns * rows, open = 0;
+    for (int q = 0; q < nq; ++q) {
+        if (q == 0 || off[q] - off[q - 1] > 16) open = q;
+        if (q == nq - 1 || off[q + 1] - off[q] > 16)
+            at += (rows + (off[q] - off[open]) + 8 + 3) / 4 * 4;
+    }
+    return at;
+}
+
+// The form itself, one row per thread, from the finished list.  A matrix whose
+// tiles would not fit in shared memory (fifteen diagonals with values of their
+// own) keeps the CSR steps: reading those from global memory took twice their
+// time.
 __global__ void __launch_bounds__(256)
 k_diag_fill(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colind,
             const float* __restrict__ vals, int32_t n, int32_t most, DiagHead* H, float* same, float* out,
             int32_t ld, void* mask, int32_t mask_bytes) {
     __shared__ int32_t s_off[DIAG_MAX];
     __shared__ unsigned s_same;
+    __shared__ bool s_bad;
     const int tid = threadIdx.x;
     if (tid < 32) {
         const int32_t o = H->off[tid];
@@ -425,11 +535,16 @@ k_diag_fill(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ coli
         for (int i = 0; i < DIAG_MAX; ++i) rank += __shfl_sync(0xffffffffu, o, i) < o;
         const bool one = used && !((H->mixed >> tid) & 1);
         const unsigned bits = __reduce_or_sync(0xffffffffu, one ? 1u << rank : 0u);
-        const bool bad = nq > most || *(volatile int32_t*)&H->w[0] != 0;
         if (used) s_off[rank] = o;
-        if (tid == 0) s_same = bad ? 0xffffffffu : bits;
+        __syncwarp();
+        const int owns = nq - __popc(bits);
+        const bool bad = nq > most || *(volatile int32_t*)&H->w[0] != 0 ||
+                         diag_room(s_off, nq, owns, DIAG_TILE) > DIAG_CAP;
+        if (tid == 0) {
+            s_same = bits;
+            s_bad = bad;
+        }
         if (blockIdx.x == 0) {
-            __syncwarp();
             if (used) {
                 H->w[4 + rank] = o;
                 if (one) same[rank] = __int_as_float((int)H->ref[tid]);
@@ -437,40 +552,31 @@ k_diag_fill(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ coli
             if (tid == 0) {
                 H->w[1] = nq;
                 H->w[2] = (int32_t)bits;
-                // two tiles at once where their windows (see diag_tile) fit
-                int at = (nq - __popc(bits)) * 2 * DIAG_TILE, open = 0;
-                for (int q = 0; q < nq; ++q) {
-                    if (q == 0 || s_off[q] - s_off[q - 1] > 16) open = q;
-                    if (q == nq - 1 || s_off[q + 1] - s_off[q] > 16)
-                        at += (2 * DIAG_TILE + (s_off[q] - s_off[open]) + 8 + 3) / 4 * 4;
-                }
-                H->w[3] = at <= DIAG_CAP;
+                H->w[3] = diag_room(s_off, nq, owns, 2 * DIAG_TILE) <= DIAG_CAP;   // two tiles at once
                 if (bad) H->w[0] = 1;
             }
         }
-        __syncwarp();
-        if (bad && tid == 0) s_off[0] = DIAG_NONE;
     }
     __syncthreads();
-    if (s_off[0] == DIAG_NONE) return;
+    if (s_bad) return;
     const unsigned same_bits = s_same;
-    const int64_t r = (int64_t)blockIdx.x * 256 + tid;
-    if (r >= n) return;
-    const int32_t e = __ldg(rowptr + r + 1);
-    unsigned bits = 0;
-    int q = 0;
-    for (int32_t k = __ldg(rowptr + r); k < e; ++k, ++q) {
-        const int32_t o = __ldg(colind + k) - (int32_t)r;
-        while (s_off[q] != o) ++q;
-        bits |= 1u << q;
-        if (!((same_bits >> q) & 1)) out[(int64_t)q * ld + r] = __ldg(vals + k);
+    for (int64_t r = (int64_t)blockIdx.x * 256 + tid; r < n; r += (int64_t)gridDim.x * 256) {
+        const int32_t e = __ldg(rowptr + r + 1);
+        unsigned bits = 0;
+        int q = 0;
+        for (int32_t k = __ldg(rowptr + r); k < e; ++k, ++q) {
+            const int32_t o = __ldg(colind + k) - (int32_t)r;
+            while (s_off[q] != o) ++q;
+            bits |= 1u << q;
+            if (!((same_bits >> q) & 1)) out[(int64_t)q * ld + r] = __ldg(vals + k);
+        }
+        if (mask_bytes == 1)
+            ((uint8_t*)mask)[r] = (uint8_t)bits;
+        else if (mask_bytes == 2)
+            ((uint16_t*)mask)[r] = (uint16_t)bits;
+        else
+            ((uint32_t*)mask)[r] = bits;
     }
-    if (mask_bytes == 1)
-        ((uint8_t*)mask)[r] = (uint8_t)bits;
-    else if (mask_bytes == 2)
-        ((uint16_t*)mask)[r] = (uint16_t)bits;
-    else
-        ((uint32_t*)mask)[r] = bits;
 }
 
 // where a tile's diagonals lie in its shared memory, in bytes
@@ -518,13 +624,12 @@ __device__ __forceinline__ bool diag_arrived(uint32_t bar) {
 // threads, thread tid on rows tid + i NT of each half.  Two at once double the
 // bytes in flight and halve what a CTA pays before its copies leave (160^3 p(A)
 // of 60 steps 1.63 -> 1.50 ms, 1500^2 0.81 -> 0.75 ms).  Warp 0 merges offsets less than 16 apart into windows
-// of x, lays windows and values out in the CAP elements of `sm`, and issues
-// the copies: values before the wait on the previous step, windows after it.
-// A tile whose data does not fit (many diagonals with values of their own)
-// reads global memory instead.
-template <typename T, int OP, int NT, int RPT, int CAP>
+// of x, lays windows and values out in `sm`, and issues
+// the copies: values before the wait on the previous step, windows after it
+// (k_diag_fill has seen to it that they fit).
+template <typename T, int OP, int NT, int RPT>
 __device__ __forceinline__ void diag_tile(const StepArgs<T>& a, int32_t row0, int nrows, float* sm,
-                                          DiagSlot* slot, uint64_t* bar, int* info, double& sq,
+                                          DiagSlot* slot, uint64_t* bar, double& sq,
                                           const int halves) {
     constexpr int HALF = NT * RPT;
     const int ROWS = HALF * halves;
@@ -567,29 +672,26 @@ __device__ __forceinline__ void diag_tile(const StepArgs<T>& a, int32_t row0, in
         const bool own = used && !((same >> lane) & 1);
         const unsigned owns = __ballot_sync(0xffffffffu, own);
         const int32_t vat = xs + __popc(owns & (upto >> 1)) * ROWS;
-        const bool fits = xs + __popc(owns) * ROWS <= CAP;
         if (used)
             slot[lane] = {(at + (int32_t)skew + (row0 + o - lo)) * 4, own ? vat * 4 : DIAG_SAME,
                           own ? 0.0f : __ldg(f.same + lane), o};
         const uint32_t bytes = opens && hi > lo ? bytes_to : 0;
         const uint32_t total = __reduce_add_sync(0xffffffffu, bytes) + __popc(owns) * (ROWS * 4u);
         if (lane == 0) {
-            info[0] = nq;
-            info[1] = fits;
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb) : "memory");
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb),
-                         "r"(fits ? total : 0u)
+                         "r"(total)
                          : "memory");
         }
         __syncwarp();
         const uint32_t base = (uint32_t)__cvta_generic_to_shared(sm);
-        if (fits && own)
+        if (own)
             bulk_to_shared(base + vat * 4, f.vals + (int64_t)lane * f.ld + row0, ROWS * 4, mb);
         // the vectors written by the previous step are complete and visible
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        if (fits && bytes) bulk_to_shared(base + at * 4, a.x + lo - (int)skew, bytes, mb);
+        if (bytes) bulk_to_shared(base + at * 4, a.x + lo - (int)skew, bytes, mb);
     } else {
         asm volatile("griddepcontrol.wait;" ::: "memory");
     }
@@ -610,7 +712,7 @@ __device__ __forceinline__ void diag_tile(const StepArgs<T>& a, int32_t row0, in
             __syncthreads();
             ready = diag_arrived(mb);
         }
-        if (ready && info[1]) {
+        if (ready) {
             // rows that lack a diagonal only where a grid ends: most warps have none
             const unsigned all = 0xffffffffu >> (32 - nq);
             bool whole = true;
@@ -638,7 +740,7 @@ __device__ __forceinline__ void diag_tile(const StepArgs<T>& a, int32_t row0, in
                             acc[i] = fma(s.v == DIAG_SAME ? s.same : at(s.v, i), at(s.x, i), acc[i]);
                 }
             }
-        } else {   // no room, or the copies did not arrive: from global memory
+        } else {   // the copies did not arrive: from global memory
             for (int q = 0; q < nq; ++q) {
                 const DiagSlot s = slot[q];
 #pragma unroll
@@ -649,7 +751,7 @@ __device__ __forceinline__ void diag_tile(const StepArgs<T>& a, int32_t row0, in
                                      __ldg(a.x + r + s.off), acc[i]);
                     }
             }
-            if (!ready) diag_arrived(mb);   // nothing may land in this CTA's memory after it
+            diag_arrived(mb);   // nothing may land in this CTA's memory after it
         }
 #pragma unroll
         for (int i = 0; i < RPT; ++i)
@@ -698,7 +800,6 @@ k_spmv_step(const StepArgs<T> a) {
         if (__ldg(a.diag.head) == 0) {   // uniform over the grid
             __shared__ __align__(16) DiagSlot slot[DIAG_MAX];
             __shared__ uint64_t bar;
-            __shared__ int info[2];
             double sq = 0.0;
             int halves = 1, rows = nrows;
             if (OP != OP_RESID && __ldg(a.diag.head + 3)) {   // two tiles on every other CTA
@@ -706,8 +807,7 @@ k_spmv_step(const StepArgs<T> a) {
                 halves = (int64_t)a.n - row0 > ROWS ? 2 : 1;
                 rows = (int)min((int64_t)a.n - row0, (int64_t)2 * ROWS);
             }
-            diag_tile<T, OP, NT, RPT, DIAG_CAP>(a, (int32_t)row0, rows, (float*)stage, slot, &bar, info,
-                                                sq, halves);
+            diag_tile<T, OP, NT, RPT>(a, (int32_t)row0, rows, (float*)stage, slot, &bar, sq, halves);
             if constexpr (OP == OP_RESID) block_sq<NT>(sq, sred, a.part);
             return;
         }
@@ -1174,10 +1274,13 @@ int32_t DiagStore::build(const int32_t* rowptr, const int32_t* colind, const flo
     f.vals = (const float*)(m + 1024);
     f.mask = m + 1024 + b_vals;
     f.ld = ld;
-    k_diag_init<<<1, 64, 0, stream>>>(H);
-    k_diag_find<<<(n + DIAG_ROWS - 1) / DIAG_ROWS, DIAG_ROWS, 0, stream>>>(rowptr, colind, vals, n,
-                                                                           most, H);
-    k_diag_fill<<<(n + 255) / 256, 256, 0, stream>>>(rowptr, colind, vals, n, most, H, (float*)f.same,
+    k_diag_init<<<1, 64, 0, stream>>>(rowptr, colind, vals, n, most, H);
+    // CTAs that stay: where there is no such form, all leave at once
+    const int sms = device_sm_count();
+    const int find = std::min((n + DIAG_ROWS - 1) / DIAG_ROWS, 10 * sms);
+    const int fill = std::min((n + 255) / 256, 8 * sms);
+    k_diag_find<<<find, DIAG_ROWS, 0, stream>>>(rowptr, colind, vals, n, most, H);
+    k_diag_fill<<<fill, 256, 0, stream>>>(rowptr, colind, vals, n, most, H, (float*)f.same,
                                                         (float*)f.vals, ld, (void*)f.mask, f.mask_bytes);
     g_launches += 3;
     PPG_TRY(check_launch("k_diag_fill"));

@@ -5,7 +5,7 @@ import pytest
 
 import synth
 from gpu_util import dev_csr, ppg_or_skip, to_dev
-from test_gpu_diagonals import CASES, GRID, _banded
+from test_gpu_diagonals import CASES, GRID, _banded, _csr_steps, _roots
 
 pytestmark = pytest.mark.gpu
 
@@ -39,6 +39,45 @@ def test_unsorted_row_has_no_diagonal_form(env):
     H.colind[[k, k + 1]] = H.colind[[k + 1, k]]
     A = p.CSR.from_host(H.rowptr, H.colind, H.vals, dtype=torch.float32, validate=False)
     assert p.chain_form(A, 33) == "staged"
+
+
+OFF27 = [i * 10000 + j * 100 + k for i in (-1, 0, 1) for j in (-1, 0, 1) for k in (-1, 0, 1)]
+
+
+@pytest.mark.parametrize("name,kw,form", [
+    # more entries to a tile of the search than it holds at once
+    ("twenty_seven_of_one_value", dict(offsets=OFF27, one_value=OFF27, n=1_300_001), "diagonals"),
+    # more values of their own than a tile's shared memory holds
+    ("thirteen_apart", CASES["thirteen_apart"], "staged"),
+    ("twenty_seven_own", dict(offsets=OFF27, n=1_300_001), "staged"),
+    # the middle row, which the list starts from, and the tiles' first rows empty
+    ("empty_rows", dict(offsets=GRID, drop=0.2, empty=[1_300_001] + list(range(0, 2_600_000, 128))),
+     "diagonals"),
+])
+def test_search_for_the_diagonals(env, name, kw, form):
+    """... and p(A) v over the form found equals the CSR steps."""
+    p, torch = env
+    A = dev_csr(p, torch, _banded(**kw), dtype=torch.float32)
+    assert p.chain_form(A, 33) == form
+    v = to_dev(torch, np.random.default_rng(4).standard_normal(A.n), torch.float32)
+    R = p.Roots.from_complex(_roots())
+    assert torch.equal(p.apply_poly(A, R, v), _csr_steps(p, torch, A, R, v))
+
+
+def test_an_offset_late_in_the_matrix(env):
+    """Rows with an offset of their own near the end: one more diagonal, or (forty
+    of them) no form; and single entries whose value differs."""
+    p, torch = env
+    R = p.Roots.from_complex(_roots())
+    v = to_dev(torch, np.random.default_rng(4).standard_normal(2_600_003), torch.float32)
+    for rows, form in ((1, "diagonals_2"), (40, "staged")):
+        H = _banded(GRID, one_value=GRID)
+        for r in range(2_500_000, 2_500_000 + rows):
+            H.colind[H.rowptr[r + 1] - 1] = 2_510_000
+        H.vals[[5, H.rowptr[2_599_000]]] = 0.125
+        A = dev_csr(p, torch, H, dtype=torch.float32)
+        assert p.chain_form(A, 33) == form
+        assert torch.equal(p.apply_poly(A, R, v), _csr_steps(p, torch, A, R, v))
 
 
 def test_small_and_l2_held_systems(env):
