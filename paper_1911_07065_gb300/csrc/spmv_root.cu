@@ -710,7 +710,8 @@ __device__ __forceinline__ void diag_tile(const StepArgs<T>& a, int32_t row0, in
         }
         if (h == 0) {
             __syncthreads();
-            ready = diag_arrived(mb);
+            // (one answer for the warp: its lanes poll apart, and vote below)
+            ready = __all_sync(0xffffffffu, diag_arrived(mb));
         }
         if (ready) {
             // rows that lack a diagonal only where a grid ends: most warps have none
