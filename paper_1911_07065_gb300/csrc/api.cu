@@ -590,9 +590,13 @@ static int32_t run_solve(SolveCore& c) {
     if (!std::isfinite(beta)) return PPG_ERR_NONFINITE;
     bool converged = c.st.true_relres <= c.tol;
 
-    if (pp && c.flex && !c.sweep && !converged)
+    if (pp && c.flex && !c.sweep && !converged) {
+        // the steps of several outer iterations, if the limits allow that many
+        const int64_t outer = std::min<int64_t>(4, (int64_t)m * (c.opts.max_cycles > 0 ? c.opts.max_cycles : 4));
         PPG_TRY(c.diag.build(c.A32->rowptr, c.A32->colind, (const float*)c.A32->vals, n, nnz,
-                             4 * (int64_t)c.p_plan.size(), s));   // (several outer steps)
+                             outer * (int64_t)c.p_plan.size(), s));
+        PPG_TRY(c.diag.settle(scal_h));
+    }
     Buffers phib{};
     phib.ptr[B_A] = c.va;
     phib.ptr[B_B] = c.vb;

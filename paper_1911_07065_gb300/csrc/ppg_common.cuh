@@ -224,9 +224,15 @@ struct DiagStore {
         if (f.head && fresh) a.flags |= F_SERIAL;
         fresh = false;
     }
-    ~DiagStore() {
+    // Wait for the search; without a form the memory goes back and the steps are
+    // the kernels that know of none.  `pinned`: room for an int32_t.
+    int32_t settle(void* pinned);
+    void drop() {
         if (mem) cudaFreeAsync(mem, s);
+        mem = nullptr;
+        f = DiagForm{};
     }
+    ~DiagStore() { drop(); }
 };
 
 // algorithmic bytes of one fused step

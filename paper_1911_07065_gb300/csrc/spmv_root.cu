@@ -1290,6 +1290,14 @@ int32_t DiagStore::build(const int32_t* rowptr, const int32_t* colind, const flo
     return PPG_OK;
 }
 
+int32_t DiagStore::settle(void* pinned) {
+    if (!f.head) return PPG_OK;
+    PPG_CUDA(cudaMemcpyAsync(pinned, f.head, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    PPG_CUDA(cudaStreamSynchronize(s));
+    if (*(const int32_t*)pinned != 0) drop();
+    return PPG_OK;
+}
+
 // Even placement of a grid of a few CTAs per SM.  Launched as programmatic
 // dependents, the next steps' CTAs take their places before a step's own are
 // done, wherever there is room, and a step then starts with two CTAs on some
