@@ -130,6 +130,7 @@ enum StepFlag : int {
     F_SERIAL = 16, // not a programmatic dependent: the first step that reads a
                    // diagonal form built by the kernel before it
     F_WIDE = 32,   // more than 5.5 entries in the average row
+    F_LONG = 64,   // ... more than LONG_AVG (spmv_root.cu)
 };
 
 // An FP32 matrix by its diagonals (spmv_root.cu), built on the device inside

@@ -185,6 +185,62 @@ __device__ __forceinline__ void long_rows(const StepArgs<T>& a, int64_t r, bool 
     }
 }
 
+// The tile's long rows with entries in a staged chunk, entries [c0, c1) at sval /
+// scol [k], in long_rows' order, into sum[row].  The rows are dealt to the CTA's NW
+// warps (a chunk holds some 26 rows of 135 entries, which are neighbours: with a
+// warp on its own 32 rows, one warp would have them all), by a hash, so that every
+// second or fourth row being long leaves none idle.  One row at most is left
+// unfinished, and its warp has it again in the next chunk: its lanes' sums stay
+// behind the rows' in sum.
+template <typename T, int NW, int ROWS>
+__device__ __forceinline__ void long_rows_staged(const int32_t* srp, const T* sval, const int32_t* scol,
+                                                 const T* __restrict__ x, int nrows, int32_t c0,
+                                                 int32_t c1, T* sum) {
+    constexpr int B = NW == 8 ? 3 : 2;
+    static_assert(NW == 1 << B, "the hash");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i0 = 0; i0 < ROWS / NW; i0 += 32) {
+        const int i = i0 + lane;
+        const int t = NW * i + (warp ^ ((i ^ (i >> B) ^ (i >> 2 * B)) & (NW - 1)));
+        bool has = false;
+        if (t < nrows) {
+            const int32_t lo = srp[t], hi = srp[t + 1];
+            has = hi - lo > LONG_ROW && lo < c1 && hi > c0;
+        }
+        unsigned todo = __ballot_sync(0xffffffffu, has);
+        while (todo) {
+            const int row = __shfl_sync(0xffffffffu, t, __ffs(todo) - 1);
+            todo &= todo - 1;
+            const int32_t lo = srp[row], hi = srp[row + 1], e = min(hi, c1);
+            int32_t k = lo + lane;
+            T part = T(0);
+            if (lo < c0) {
+                part = sum[ROWS + lane];
+                k += (c0 - lo - lane + 31) / 32 * 32;   // (0 where the lane has had none)
+            }
+            for (; k < e; k += 128) {
+                T v[4], g[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (k + 32 * u < e) {
+                        v[u] = sval[k + 32 * u];
+                        g[u] = __ldg(x + scol[k + 32 * u]);
+                    }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (k + 32 * u < e) part = fma(v[u], g[u], part);
+            }
+            if (hi > c1) {
+                sum[ROWS + lane] = part;
+            } else {
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
+                if (lane == 0) sum[row] = part;
+            }
+        }
+    }
+}
+
 // part[block] = the sum of sq over the CTA's NT threads, in a fixed order
 template <int NT>
 __device__ __forceinline__ void block_sq(double sq, double* sred, double* part) {
@@ -227,11 +283,24 @@ __host__ __device__ constexpr int step_min_ctas() {
     return sizeof(T) == 4 ? (OP == OP_PHI_PAIR2 ? 6 : 7) : 16;
 }
 
-// ... and of the form that also knows the diagonal steps: 40 registers, for the
-// sake of a matrix without that form, which runs its CSR part (seven random
-// entries per row, 60 steps, 2e6 rows: 2.12 ms with 7 CTAs, 1.89 with 6; the
-// kernel without diagonals 2.05).
-constexpr int DIAG_CTAS = 6;
+// ... and of the forms that also know the diagonal steps, or rows of many entries:
+// 40 registers, for the sake of their CSR part (seven random entries per row, 60
+// steps, 2e6 rows: 2.12 ms with 7 CTAs, 1.89 with 6; the plain kernel 2.05.  Rows
+// of 130 - 140 entries, 400,000 of them: 172 us a step with 7 CTAs, 135 with 6).
+constexpr int WIDE_CTAS = 6;
+
+// FP32 matrices of more entries than this in the average row take the form that
+// sums long rows from the staged chunks: of such a matrix they may be most of the
+// bytes, and read twice (long_rows) they made a step up to 1.5 times as long as with
+// one thread to a row.  400,000 rows of 130 - 140 entries: one thread 162 us a
+// step, read twice 235, from the chunks 135; every fourth row of 140, the others of
+// 3: 107, 153 and 82; every eighth 103, 113 and 65; every sixteenth (11.6 in the
+// average row) 96 and 55, read twice.  Without long rows the form costs its two
+// registers: 30 entries in every row 90.7 -> 92.1 us, 45 99.9 -> 102.2, 100 112 ->
+// 99.  In FP64 a long row is bound by its multiply-adds, and reading it twice is
+// faster than one thread throughout (the same matrices: 583 -> 350, 485 -> 237, 518
+// -> 164 us), so FP64 has no such form: it cost the steps of grids 10 %.
+constexpr double LONG_AVG = 16.0;
 
 // one row's multiply-adds over its staged nonzeros [lo, hi): four gathers in
 // flight, then the last 1-3 (FP32: issued together; FP64: one at a time)
@@ -768,11 +837,60 @@ __device__ __forceinline__ void diag_tile(const StepArgs<T>& a, int32_t row0, in
     }
 }
 
-// PF: prefetch the tile a.pf_ahead tiles ahead (half a resident wave) into
-// L2 (launched when the matrix is not held in an L2 set-aside)
+// A tile of k_spmv_step that has long rows, its row pointers in srp: ordinary rows
+// by a thread each, long rows from the staged chunks.
+template <typename T, int OP>
+__device__ __forceinline__ double long_tile(const StepArgs<T>& a, int64_t row0, int nrows, T* sval,
+                                            int32_t* scol, const int32_t* srp) {
+    constexpr int NT = step_threads<T>(), RPT = step_rpt<T>(), ROWS = NT * RPT;
+    constexpr int CHUNK = step_chunk<T>() - ROWS - 32;   // the long rows' sums lie behind it
+    static_assert(CHUNK % 4 == 0, "16-byte granules");
+    T* const sum = sval + CHUNK + 4;
+    const int tid = threadIdx.x;
+    const int32_t k0 = srp[0], k1 = srp[nrows];
+    T acc[RPT];
+#pragma unroll
+    for (int q = 0; q < RPT; ++q) acc[q] = T(0);
+    for (int32_t c0 = k0, c1; c0 < k1; c0 = c1) {
+        c1 = c0 + min(k1 - c0, CHUNK);
+        const int32_t base = c0 & ~3;
+        if (c0 != k0) __syncthreads();
+        stage_chunk<T>(sval, scol, a.vals, a.colind, base, c0, c1, tid, NT,
+                       l2_policy((a.flags & F_KEEP_A) || row0 < a.keep_rows));
+        // the vectors written by the previous step are complete and visible
+        if (c0 == k0) asm volatile("griddepcontrol.wait;" ::: "memory");
+        cp_async_wait_all();
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < RPT; ++q) {
+            const int t = tid + q * NT;
+            if (t < nrows && srp[t + 1] - srp[t] <= LONG_ROW)
+                acc[q] = row_dot<T, true>(sval, scol, a.x, max(srp[t], c0) - base,
+                                          min(srp[t + 1], c1) - base, acc[q]);
+        }
+        long_rows_staged<T, NT / 32, ROWS>(srp, sval - base, scol - base, a.x, nrows, c0, c1, sum);
+    }
+    __syncthreads();
+    double sq = 0.0;
+#pragma unroll
+    for (int q = 0; q < RPT; ++q) {
+        const int t = tid + q * NT;
+        if (t < nrows) {
+            const int64_t r = row0 + t;
+            const T e0 = a.a0 ? __ldg(a.a0 + r) : T(0);
+            const T e1 = (a.a1 && !(a.flags & F_PZERO)) ? a.a1[r] : T(0);
+            const T e2 = (a.a2 && (a.flags & F_FINAL)) ? __ldg(a.a2 + r) : T(0);
+            step_epilogue<T, OP>(a, r, srp[t + 1] - srp[t] > LONG_ROW ? sum[t] : acc[q], e0, e1, e2, sq);
+        }
+    }
+    return sq;
+}
+
 // DG: the (FP32) matrix is at hand by its diagonals too, if it has that form
-template <typename T, int OP, bool PF, bool DG>
-__global__ void __launch_bounds__(step_threads<T>(), DG ? DIAG_CTAS : step_min_ctas<T, OP>())
+// LR: a tile with long rows sums them from its staged chunks (long_tile), else they
+// are read a second time (long_rows)
+template <typename T, int OP, bool DG, bool LR>
+__global__ void __launch_bounds__(step_threads<T>(), DG || LR ? WIDE_CTAS : step_min_ctas<T, OP>())
 k_spmv_step(const StepArgs<T> a) {
     constexpr int NT = step_threads<T>();      // threads per CTA
     // staging copies start at a chunk base rounded down to 4 elements
@@ -820,15 +938,29 @@ k_spmv_step(const StepArgs<T> a) {
     int64_t prow = row0 + (int64_t)a.pf_ahead * ROWS;
     const bool wrap = prow >= a.n;
     if (wrap) prow -= (int64_t)gridDim.x * ROWS;
-    const bool pf = PF && tid == 0 && a.pf_ahead > 0 && prow >= 0 && prow < a.n;
+    const bool pf = tid == 0 && a.pf_ahead > 0 && prow >= 0 && prow < a.n;
     const int64_t prow1 = min(prow + ROWS, (int64_t)a.n);
     int32_t pk0 = 0, pk1 = 0;
     if (pf) {
         pk0 = __ldg(a.rowptr + prow);
         pk1 = __ldg(a.rowptr + prow1);
     }
-    for (int i = tid; i <= nrows; i += NT) srp[i] = __ldg(a.rowptr + row0 + i);
-    __syncthreads();
+    if constexpr (LR) {
+        bool any = false;
+        for (int i = tid; i <= nrows; i += NT) {
+            const int32_t k = __ldg(a.rowptr + row0 + i);
+            srp[i] = k;
+            any = any || (i < nrows && __ldg(a.rowptr + row0 + i + 1) - k > LONG_ROW);
+        }
+        if (__syncthreads_or(any)) {
+            const double sq = long_tile<T, OP>(a, row0, nrows, sval, scol, srp);
+            if constexpr (OP == OP_RESID) block_sq<NT>(sq, sred, a.part);
+            return;
+        }
+    } else {
+        for (int i = tid; i <= nrows; i += NT) srp[i] = __ldg(a.rowptr + row0 + i);
+        __syncthreads();
+    }
     const int32_t k0 = srp[0];
     const int32_t k1 = srp[nrows];
     // thread tid owns rows tid and (RPT = 2) tid + NT of the tile
@@ -839,7 +971,7 @@ k_spmv_step(const StepArgs<T> a) {
         const int t = tid + q * NT;
         my_lo[q] = (t < nrows) ? srp[t] : k1;
         my_hi[q] = (t < nrows) ? srp[t + 1] : k1;
-        is_long[q] = my_hi[q] - my_lo[q] > LONG_ROW;
+        is_long[q] = !LR && my_hi[q] - my_lo[q] > LONG_ROW;
         if (is_long[q]) my_hi[q] = my_lo[q];   // (long_rows below)
     }
     // element k of the current chunk sits at sval / scol [k - base], base =
@@ -931,8 +1063,10 @@ k_spmv_step(const StepArgs<T> a) {
         if (t < nrows && !is_long[q])
             step_epilogue<T, OP>(a, row0 + t, acc[q], e0[q], e1[q], e2[q], sq);
     }
+    if constexpr (!LR) {
 #pragma unroll
-    for (int q = 0; q < RPT; ++q) long_rows<T, OP>(a, row0 + tid + q * NT, is_long[q], sq);
+        for (int q = 0; q < RPT; ++q) long_rows<T, OP>(a, row0 + tid + q * NT, is_long[q], sq);
+    }
     if constexpr (OP == OP_RESID) block_sq<NT>(sq, sred, a.part);
 }
 
@@ -1192,31 +1326,32 @@ int keep_a_flag(int64_t n, int64_t nnz, int elem, int nvec, bool may_reserve,
     if (l2 <= 0 || n <= 0) return 0;
     const double a_bytes = (double)nnz * (elem + 4) + 4.0 * (n + 1);
     const double bytes = a_bytes + (double)nvec * n * elem;
+    const int rows = ((double)nnz > 5.5 * (double)n ? F_WIDE : 0) |
+                     ((double)nnz > LONG_AVG * (double)n ? F_LONG : 0);
     if (!fits_l2(bytes, l2)) {
         // streaming: a chain holds the nonzeros of its leading rows in a
         // set-aside of kPartialL2 (shrinking a larger one that an L2-resident
         // workload left: an unused 76 MB set-aside cost the 160^3 FP32 chains
         // 11 %), and streams the rest
-        if (!keep_rows) return 0;
+        if (!keep_rows) return rows;
         const size_t have = may_reserve ? set_l2_exact(dev, kPartialL2)
                                         : g_l2_reserved[dev].load(std::memory_order_relaxed);
-        const double rows = 0.9 * (double)have / (a_bytes / (double)n);
-        *keep_rows = (int32_t)(rows < (double)n ? rows : (double)n);
-        return 0;
+        const double held = 0.9 * (double)have / (a_bytes / (double)n);
+        *keep_rows = (int32_t)(held < (double)n ? held : (double)n);
+        return rows;
     }
     const size_t need = (size_t)(a_bytes * 1.05);
-    const int wide = (double)nnz > 5.5 * (double)n ? F_WIDE : 0;
     if (may_reserve) {
         reserve_l2_for(dev, need);
-        return F_KEEP_A | wide;
+        return F_KEEP_A | rows;
     }
     // no change to the context: the hint only where a set-aside exists
-    return g_l2_reserved[dev].load(std::memory_order_relaxed) >= need ? F_KEEP_A | wide : 0;
+    return rows | (g_l2_reserved[dev].load(std::memory_order_relaxed) >= need ? F_KEEP_A : 0);
 }
 
 // CTAs of the root-step kernel resident at once (occupancy x SMs), per
-// device and element type
-template <typename T>
+// device and form of the kernel
+template <typename T, bool DG, bool LR>
 static int step_resident_ctas() {
     static std::atomic<int> cached[16];
     int dev = 0;
@@ -1224,7 +1359,7 @@ static int step_resident_ctas() {
     int v = cached[dev].load(std::memory_order_relaxed);
     if (v == 0) {
         int occ = 0, sms = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_spmv_step<T, OP_P_REAL, true, false>,
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_spmv_step<T, OP_P_REAL, DG, LR>,
                                                           step_threads<T>(), 0) != cudaSuccess ||
             occ < 1)
             occ = 1;
@@ -1353,16 +1488,16 @@ static cudaError_t launch_direct(cudaLaunchConfig_t& cfg, int op, const StepArgs
     }
 }
 
-template <typename T, bool PF, bool DG>
+template <typename T, bool DG, bool LR>
 static cudaError_t launch_op(cudaLaunchConfig_t& cfg, int op, const StepArgs<T>& a) {
     switch (op) {
-        case OP_SPMV: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_SPMV, PF, DG>, a);
-        case OP_RESID: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_RESID, PF, DG>, a);
-        case OP_PHI_REAL: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_PHI_REAL, PF, DG>, a);
-        case OP_PHI_PAIR2: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_PHI_PAIR2, PF, DG>, a);
-        case OP_P_REAL: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_P_REAL, PF, DG>, a);
-        case OP_P_PAIR1: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_P_PAIR1, PF, DG>, a);
-        case OP_P_PAIR2: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_P_PAIR2, PF, DG>, a);
+        case OP_SPMV: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_SPMV, DG, LR>, a);
+        case OP_RESID: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_RESID, DG, LR>, a);
+        case OP_PHI_REAL: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_PHI_REAL, DG, LR>, a);
+        case OP_PHI_PAIR2: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_PHI_PAIR2, DG, LR>, a);
+        case OP_P_REAL: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_P_REAL, DG, LR>, a);
+        case OP_P_PAIR1: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_P_PAIR1, DG, LR>, a);
+        case OP_P_PAIR2: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_P_PAIR2, DG, LR>, a);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -1378,7 +1513,12 @@ int32_t launch_step(int op, const StepArgs<T>& a_in, cudaStream_t s) {
     // 3-D 160^3 chains (FP32 / FP64) by distance in resident waves:
     // 1/4 5860 / 6121 GB/s, 1/3 6017 / 6141, 1/2 6041 / 6151, 1 5969 / 6142,
     // 3/2 5836 / 6123, 2 5218 / 5982.
-    a.pf_ahead = (a.flags & F_KEEP_A) ? 0 : (step_resident_ctas<T>() + 1) / 2;
+    constexpr bool F32 = sizeof(T) == 4;
+    const bool dg = F32 && a.diag.head != nullptr, lr = F32 && (a.flags & F_LONG);
+    a.pf_ahead = (a.flags & F_KEEP_A) ? 0
+                 : ((lr ? (dg ? step_resident_ctas<T, F32, F32>() : step_resident_ctas<T, false, F32>())
+                        : (dg ? step_resident_ctas<T, F32, false>() : step_resident_ctas<T, false, false>())) +
+                    1) / 2;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(step_threads<T>());
@@ -1391,8 +1531,6 @@ int32_t launch_step(int op, const StepArgs<T>& a_in, cudaStream_t s) {
     cfg.numAttrs = (a.flags & F_SERIAL) ? 0 : 1;
     if (op < OP_SPMV || op > OP_P_PAIR2) return PPG_ERR_ARG;
     const bool small = a_in.n <= DIRECT_MAX_N;
-    constexpr bool F32 = sizeof(T) == 4;
-    const bool dg = F32 && a.diag.head != nullptr;
     if (small || ((a_in.flags & F_KEEP_A) && !dg)) {
         // one row per thread, no staging round (small system, or matrix in L2)
         const int dgrid = (int)(((int64_t)a_in.n + SPMV_ROWS - 1) / SPMV_ROWS);
@@ -1444,7 +1582,8 @@ int32_t launch_step(int op, const StepArgs<T>& a_in, cudaStream_t s) {
         return dgrid;
     }
     const cudaError_t e =
-        dg ? launch_op<T, true, F32>(cfg, op, a) : launch_op<T, true, false>(cfg, op, a);
+        lr ? (dg ? launch_op<T, F32, F32>(cfg, op, a) : launch_op<T, false, F32>(cfg, op, a))
+           : (dg ? launch_op<T, F32, false>(cfg, op, a) : launch_op<T, false, false>(cfg, op, a));
     ++g_launches;
     if (e != cudaSuccess) {
         set_cuda_error(e, "cudaLaunchKernelEx(k_spmv_step)");
