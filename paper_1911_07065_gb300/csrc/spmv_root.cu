@@ -777,22 +777,23 @@ __device__ __forceinline__ void diag_tile(const StepArgs<T>& a, int32_t row0, in
                 if (a.a2 && (a.flags & F_FINAL)) e2[i] = __ldg(a.a2 + r);
             }
         }
+        // rows that lack a diagonal only where a grid ends: most warps have none
+        const unsigned all = 0xffffffffu >> (32 - nq);
+        bool whole = true;
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) whole = whole && b[i] == all;
+        whole = __all_sync(0xffffffffu, whole);
         if (h == 0) {
             __syncthreads();
-            // (one answer for the warp: its lanes poll apart, and vote below)
+            // (one answer for the warp: its lanes poll apart, the sums below are the warp's)
             ready = __all_sync(0xffffffffu, diag_arrived(mb));
         }
         if (ready) {
-            // rows that lack a diagonal only where a grid ends: most warps have none
-            const unsigned all = 0xffffffffu >> (32 - nq);
-            bool whole = true;
-#pragma unroll
-            for (int i = 0; i < RPT; ++i) whole = whole && b[i] == all;
             const char* me = reinterpret_cast<const char*>(sm + tid);
             auto at = [&](int32_t off, int i) {
                 return *reinterpret_cast<const float*>(me + off + i * NT * (int)sizeof(float));
             };
-            if (__all_sync(0xffffffffu, whole)) {
+            if (whole) {
 #pragma unroll 4
                 for (int q = 0; q < nq; ++q) {
                     const DiagSlot s = slot[q];
