@@ -190,12 +190,12 @@ __device__ __forceinline__ void long_rows(const StepArgs<T>& a, int64_t r, bool 
 // warps (a chunk holds some 26 rows of 135 entries, which are neighbours: with a
 // warp on its own 32 rows, one warp would have them all), by a hash, so that every
 // second or fourth row being long leaves none idle.  One row at most is left
-// unfinished, and its warp has it again in the next chunk: its lanes' sums stay
-// behind the rows' in sum.
+// unfinished, and its warp has it again in the next chunk: its lanes' sums go to
+// `left`, and come from `from`, which another warp's row may have to itself by then.
 template <typename T, int NW, int ROWS>
 __device__ __forceinline__ void long_rows_staged(const int32_t* srp, const T* sval, const int32_t* scol,
                                                  const T* __restrict__ x, int nrows, int32_t c0,
-                                                 int32_t c1, T* sum) {
+                                                 int32_t c1, T* sum, const T* from, T* left) {
     constexpr int B = NW == 8 ? 3 : 2;
     static_assert(NW == 1 << B, "the hash");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -215,7 +215,7 @@ __device__ __forceinline__ void long_rows_staged(const int32_t* srp, const T* sv
             int32_t k = lo + lane;
             T part = T(0);
             if (lo < c0) {
-                part = sum[ROWS + lane];
+                part = from[lane];
                 k += (c0 - lo - lane + 31) / 32 * 32;   // (0 where the lane has had none)
             }
             for (; k < e; k += 128) {
@@ -231,7 +231,7 @@ __device__ __forceinline__ void long_rows_staged(const int32_t* srp, const T* sv
                     if (k + 32 * u < e) part = fma(v[u], g[u], part);
             }
             if (hi > c1) {
-                sum[ROWS + lane] = part;
+                left[lane] = part;
             } else {
 #pragma unroll
                 for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
@@ -844,7 +844,7 @@ template <typename T, int OP>
 __device__ __forceinline__ double long_tile(const StepArgs<T>& a, int64_t row0, int nrows, T* sval,
                                             int32_t* scol, const int32_t* srp) {
     constexpr int NT = step_threads<T>(), RPT = step_rpt<T>(), ROWS = NT * RPT;
-    constexpr int CHUNK = step_chunk<T>() - ROWS - 32;   // the long rows' sums lie behind it
+    constexpr int CHUNK = step_chunk<T>() - ROWS - 64;   // the long rows' sums lie behind it
     static_assert(CHUNK % 4 == 0, "16-byte granules");
     T* const sum = sval + CHUNK + 4;
     const int tid = threadIdx.x;
@@ -852,6 +852,7 @@ __device__ __forceinline__ double long_tile(const StepArgs<T>& a, int64_t row0, 
     T acc[RPT];
 #pragma unroll
     for (int q = 0; q < RPT; ++q) acc[q] = T(0);
+    T *from = sum + ROWS, *left = from + 32;
     for (int32_t c0 = k0, c1; c0 < k1; c0 = c1) {
         c1 = c0 + min(k1 - c0, CHUNK);
         const int32_t base = c0 & ~3;
@@ -869,7 +870,10 @@ __device__ __forceinline__ double long_tile(const StepArgs<T>& a, int64_t row0, 
                 acc[q] = row_dot<T, true>(sval, scol, a.x, max(srp[t], c0) - base,
                                           min(srp[t + 1], c1) - base, acc[q]);
         }
-        long_rows_staged<T, NT / 32, ROWS>(srp, sval - base, scol - base, a.x, nrows, c0, c1, sum);
+        long_rows_staged<T, NT / 32, ROWS>(srp, sval - base, scol - base, a.x, nrows, c0, c1, sum, from, left);
+        T* const was = from;
+        from = left;
+        left = was;
     }
     __syncthreads();
     double sq = 0.0;

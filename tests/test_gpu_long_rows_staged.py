@@ -58,6 +58,27 @@ def test_staged_equals_direct(env, name, per_row, dtype):
         assert torch.equal(p.apply_phi(big, R, vb)[: A.n], p.apply_phi(A, R, v))
 
 
+@pytest.mark.parametrize("name", ["every_fourth", "most"])
+def test_rows_over_chunk_ends_many_times(env, name):
+    """Every chunk ends within a long row and begins within another's rest, which
+    two warps have at the same time."""
+    p, torch = env
+    A = dev_csr(p, torch, random_csr(seed=3, **HEADS[name]), dtype=torch.float32)
+    v = to_dev(torch, np.random.default_rng(9).standard_normal(A.n), torch.float32)
+    k = 60
+    off = torch.arange(k, device="cuda").repeat_interleave(A.nnz)
+    rp = torch.cat([A.rowptr[:-1].long().repeat(k) + torch.arange(k, device="cuda").repeat_interleave(A.n) * A.nnz,
+                    torch.tensor([k * A.nnz], device="cuda")])
+    copies = p.CSR(rp.int(), (A.colind.long().repeat(k) + off * A.n).int(), A.vals.repeat(k))
+    big = _streamed(p, torch, copies, 20)
+    R = p.Roots.from_complex(ROOTS)
+    ref = p.apply_phi(A, R, v).repeat(k)
+    vb = torch.cat([v.repeat(k), torch.ones(big.n - copies.n, dtype=torch.float32, device="cuda")])
+    assert p.chain_form(big, 7) == "staged"
+    for _ in range(20):
+        assert torch.equal(p.apply_phi(big, R, vb)[: copies.n], ref)
+
+
 @pytest.mark.parametrize("per_row", [5, 150])
 def test_residual_with_long_rows(env, per_row):
     """The residual's norm: one cycle of one step from x0, against the residual
