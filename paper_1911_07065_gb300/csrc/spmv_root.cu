@@ -1112,6 +1112,7 @@ __device__ __forceinline__ int32_t ld_hint<int32_t>(const int32_t* p, uint64_t p
 
 constexpr int DIRECT_SMALL_ROWS = 64;   // rows (threads) per CTA, up to one such CTA per SM
 constexpr int DIRECT_L2_ROWS = 128;     // ... above that
+constexpr int LATE_MAX = 10;            // (launch_step)
 
 template <typename T, int OP, int PRE, int MINB, bool HINT>
 __global__ void __launch_bounds__(SPMV_ROWS, MINB)
@@ -1120,7 +1121,8 @@ k_spmv_direct(const StepArgs<T> a) {
     const int tid = threadIdx.x;
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + tid;
     const bool live = r < a.n;
-    asm volatile("griddepcontrol.launch_dependents;");
+    const bool late = a.flags & F_LATE;
+    if (!late) asm volatile("griddepcontrol.launch_dependents;");
     int32_t k0 = 0, k1 = 0;
     T pv[PRE];
     int32_t pc[PRE];
@@ -1142,6 +1144,7 @@ k_spmv_direct(const StepArgs<T> a) {
     }
     // the vectors written by the previous step are complete and visible
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (late) asm volatile("griddepcontrol.launch_dependents;");
     double sq = 0.0;
     const bool is_long = k1 - k0 > LONG_ROW;
     if (live) {
@@ -1438,57 +1441,16 @@ int32_t DiagStore::settle(void* pinned) {
     return PPG_OK;
 }
 
-// Even placement of a grid of a few CTAs per SM.  Launched as programmatic
-// dependents, the next steps' CTAs take their places before a step's own are
-// done, wherever there is room, and a step then starts with two CTAs on some
-// SMs and none on others.  Dynamic shared memory that nothing uses leaves each
-// SM room for its share alone: 40 FP64 steps on a grid of 150^2 156 -> 83 us,
-// 240^2 174 -> 88 us, 400^2 185 -> 148 us, on 30^3 159 -> 83 us.  It takes the
-// room from L1, so not above EVEN_MAX CTAs per SM (512^2, 14 per SM: 198 -> 205
-// us), and a grid of no more CTAs than half the SMs needs none of it (50^2: 82 -> 87
-// us).
-constexpr int EVEN_MAX = 10;
-static size_t even_smem(unsigned grid, int sms, int most) {
-    const int per = (int)((grid + sms - 1) / sms);
-    if (per > most || 2 * grid <= (unsigned)sms) return 0;
-    // 228 KB per SM, 1 KB of it taken by each CTA beside its own; a share and
-    // one CTA more must not fit
-    return (size_t)min(228 / per - 2, 116) * 1024;
-}
-
-template <typename T, int OP, int PRE, int MINB, bool HINT>
-static cudaError_t launch_even(cudaLaunchConfig_t& cfg, const StepArgs<T>& a, int most) {
-    auto kernel = k_spmv_direct<T, OP, PRE, MINB, HINT>;
-    static std::atomic<uint64_t> allowed{0};   // devices on which it may have more than 48 KB
-    size_t smem = even_smem(cfg.gridDim.x, a.sms, most);
-    if (smem > 48 * 1024) {
-        const int dev = current_device();
-        const uint64_t bit = dev < 0 ? 0 : 1ull << dev;
-        if (!(allowed.load(std::memory_order_relaxed) & bit)) {
-            if (dev >= 0 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 116 * 1024) == cudaSuccess) {
-                allowed.fetch_or(bit, std::memory_order_relaxed);
-            } else {
-                cudaGetLastError();
-                smem = 0;
-            }
-        }
-    }
-    cfg.dynamicSmemBytes = smem;
-    return cudaLaunchKernelEx(&cfg, kernel, a);
-}
-
-// most: CTAs per SM up to which they are placed evenly (0: as they come)
 template <typename T, int PRE, int MINB, bool HINT>
-static cudaError_t launch_direct(cudaLaunchConfig_t& cfg, int op, const StepArgs<T>& a, int most) {
+static cudaError_t launch_direct(cudaLaunchConfig_t& cfg, int op, const StepArgs<T>& a) {
     switch (op) {
-        case OP_SPMV: return launch_even<T, OP_SPMV, PRE, MINB, HINT>(cfg, a, most);
-        case OP_RESID: return launch_even<T, OP_RESID, PRE, MINB, HINT>(cfg, a, most);
-        case OP_PHI_REAL: return launch_even<T, OP_PHI_REAL, PRE, MINB, HINT>(cfg, a, most);
-        case OP_PHI_PAIR2: return launch_even<T, OP_PHI_PAIR2, PRE, MINB, HINT>(cfg, a, most);
-        case OP_P_REAL: return launch_even<T, OP_P_REAL, PRE, MINB, HINT>(cfg, a, most);
-        case OP_P_PAIR1: return launch_even<T, OP_P_PAIR1, PRE, MINB, HINT>(cfg, a, most);
-        case OP_P_PAIR2: return launch_even<T, OP_P_PAIR2, PRE, MINB, HINT>(cfg, a, most);
+        case OP_SPMV: return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_SPMV, PRE, MINB, HINT>, a);
+        case OP_RESID: return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_RESID, PRE, MINB, HINT>, a);
+        case OP_PHI_REAL: return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_PHI_REAL, PRE, MINB, HINT>, a);
+        case OP_PHI_PAIR2: return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_PHI_PAIR2, PRE, MINB, HINT>, a);
+        case OP_P_REAL: return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_P_REAL, PRE, MINB, HINT>, a);
+        case OP_P_PAIR1: return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_P_PAIR1, PRE, MINB, HINT>, a);
+        case OP_P_PAIR2: return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_P_PAIR2, PRE, MINB, HINT>, a);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -1551,8 +1513,19 @@ int32_t launch_step(int op, const StepArgs<T>& a_in, cudaStream_t s) {
             const int rows_d = a_in.n <= sms * DIRECT_SMALL_ROWS ? DIRECT_SMALL_ROWS : DIRECT_L2_ROWS;
             cfg.blockDim = dim3(rows_d);
             cfg.gridDim = dim3((unsigned)(((int64_t)a_in.n + rows_d - 1) / rows_d));
+            // The next step is let in by a grid of at most LATE_MAX CTAs per SM only
+            // when the previous one is done, by a larger one at once.  At once, the
+            // CTAs of a third and fourth step come in too wherever there is room, to
+            // wait there, and a small step then starts with several CTAs on some SMs
+            // and none on others.  40 FP64 steps at once / so: 2-D 150^2 155 / 85 us,
+            // 240^2 217 / 103, 300^2 216 / 135, 400^2 223 / 163; four such chains on
+            // four streams, as graphs: 300^2 182 / 178 us, 400^2 316 / 315.  (Shared
+            // memory that leaves an SM room for its share only takes 104 and 147 us
+            // for one chain of 300^2 and 400^2, but 259 and 317 for the four of them,
+            // at 240^2 250 instead of 131.)  500^2 in FP32, 13 CTAs per SM, loses by
+            // it: 116 -> 121 us.
+            if (cfg.gridDim.x <= (unsigned)(LATE_MAX * sms)) a.flags |= F_LATE;
         }
-        const int most = op == OP_RESID ? 0 : EVEN_MAX;
         // matrix in L2: entries preloaded before the dependency wait.
         // Up to 5.5 in the average row, five: FP64 at 40 registers (1536 threads
         // per SM), the plain SpMV step at 32 (2048 threads; it fits), FP32 at 40
@@ -1569,15 +1542,15 @@ int32_t launch_step(int op, const StepArgs<T>& a_in, cudaStream_t s) {
         // (45^3 201 -> 137 us, seven 146 us; 53^3 247 -> 168 us, seven 203 us).
         cudaError_t ed;
         if (small)
-            ed = launch_direct<T, 8, 0, false>(cfg, op, a, most);
+            ed = launch_direct<T, 8, 0, false>(cfg, op, a);
         else if ((a_in.flags & F_WIDE) && !F32 && a_in.n <= sms * 8 * DIRECT_L2_ROWS)
-            ed = launch_direct<T, 8, 4, true>(cfg, op, a, min(most, 6));   // (above, registers do it)
+            ed = launch_direct<T, 8, 4, true>(cfg, op, a);
         else if (a_in.flags & F_WIDE)
-            ed = launch_direct<T, 7, 6, true>(cfg, op, a, most);
+            ed = launch_direct<T, 7, 6, true>(cfg, op, a);
         else if (!F32 && op == OP_SPMV)
-            ed = launch_even<T, OP_SPMV, 5, 8, true>(cfg, a, most);
+            ed = cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_SPMV, 5, 8, true>, a);
         else
-            ed = launch_direct<T, 5, 6, true>(cfg, op, a, most);
+            ed = launch_direct<T, 5, 6, true>(cfg, op, a);
         ++g_launches;
         if (ed != cudaSuccess) {
             set_cuda_error(ed, "cudaLaunchKernelEx(k_spmv_direct)");
