@@ -185,6 +185,48 @@ __device__ __forceinline__ void long_rows(const StepArgs<T>& a, int64_t r, bool 
     }
 }
 
+// The same as a call, eight entries a lane at a time, for small systems: inlined,
+// code that few of them need costs a chain of short steps instruction fetches
+// (as a graph, 40 FP64 steps of p(A) at 100^2: 63 us without it, 76 with long_rows,
+// 68 with the call).
+template <typename T, int OP>
+__device__ __noinline__ double long_rows_call(const StepArgs<T>& a, int32_t r, unsigned todo) {
+    constexpr int U = 8;
+    const int lane = threadIdx.x & 31;
+    double sq = 0.0;
+    while (todo) {
+        const int src = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const int32_t row = __shfl_sync(0xffffffffu, r, src);
+        const int32_t k1 = __ldg(a.rowptr + row + 1);
+        T acc = T(0);
+        for (int32_t k = __ldg(a.rowptr + row) + lane; k < k1; k += 32 * U) {
+            int32_t c[U];
+            T v[U], g[U];
+            // (past the end: the last entry again, so that the loads need no branch)
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                c[u] = __ldg(a.colind + min(k + 32 * u, k1 - 1));
+                v[u] = __ldg(a.vals + min(k + 32 * u, k1 - 1));
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) g[u] = __ldg(a.x + c[u]);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (k + 32 * u < k1) acc = fma(v[u], g[u], acc);
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+        if (lane == src) {
+            const T e0 = a.a0 ? __ldg(a.a0 + r) : T(0);
+            const T e1 = (a.a1 && !(a.flags & F_PZERO)) ? a.a1[r] : T(0);
+            const T e2 = (a.a2 && (a.flags & F_FINAL)) ? __ldg(a.a2 + r) : T(0);
+            step_epilogue<T, OP>(a, r, acc, e0, e1, e2, sq);
+        }
+    }
+    return sq;
+}
+
 // The tile's long rows with entries in a staged chunk, entries [c0, c1) at sval /
 // scol [k], in long_rows' order, into sum[row].  The rows are dealt to the CTA's NW
 // warps (a chunk holds some 26 rows of 135 entries, which are neighbours: with a
@@ -1112,15 +1154,28 @@ __device__ __forceinline__ int32_t ld_hint<int32_t>(const int32_t* p, uint64_t p
 
 constexpr int DIRECT_SMALL_ROWS = 64;   // rows (threads) per CTA, up to one such CTA per SM
 constexpr int DIRECT_L2_ROWS = 128;     // ... above that
+// Rows of many entries in a small system: SPREAD_ROWS of them to a warp, so that
+// there are more warps, and that a warp with long rows has fewer to sum in turn (40
+// FP64 steps, 32 rows to a warp / 4: 400 rows of 150 1450 / 346 us, with one thread
+// to a row 477; 1,000 of 60 232 / 199; 2,500 of 24 142 / 116; below that it loses: FP32,
+// 10,000 of 18 89 / 110).
+constexpr int SPREAD_ROWS = 4;
+constexpr double SPREAD_AVG = 22.0;
 constexpr int LATE_MAX = 10;            // (launch_step)
 
 template <typename T, int OP, int PRE, int MINB, bool HINT>
 __global__ void __launch_bounds__(SPMV_ROWS, MINB)
-k_spmv_direct(const StepArgs<T> a) {
+k_spmv_direct(const __grid_constant__ StepArgs<T> a) {
     __shared__ double sred[SPMV_ROWS / 32];
     const int tid = threadIdx.x;
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + tid;
-    const bool live = r < a.n;
+    // a row to a lane; rows of many entries, in a small system, to the first few
+    // lanes of a warp (launch_step)
+    int64_t r = (int64_t)blockIdx.x * blockDim.x + tid;
+    bool live = r < a.n;
+    if (!HINT && OP != OP_RESID && (a.flags & F_SPREAD)) {
+        r = (r >> 5) * SPREAD_ROWS + (tid & 31);
+        live = (tid & 31) < SPREAD_ROWS && r < a.n;
+    }
     const bool late = a.flags & F_LATE;
     if (!late) asm volatile("griddepcontrol.launch_dependents;");
     int32_t k0 = 0, k1 = 0;
@@ -1142,6 +1197,7 @@ k_spmv_direct(const StepArgs<T> a) {
             }
         }
     }
+    const unsigned longs = HINT ? 0 : __ballot_sync(0xffffffffu, k1 - k0 > LONG_ROW);
     // the vectors written by the previous step are complete and visible
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (late) asm volatile("griddepcontrol.launch_dependents;");
@@ -1166,7 +1222,11 @@ k_spmv_direct(const StepArgs<T> a) {
             acc = fma(__ldg(a.vals + k), __ldg(a.x + __ldg(a.colind + k)), acc);
         if (!is_long) step_epilogue<T, OP>(a, r, acc, e0, e1, e2, sq);
     }
-    long_rows<T, OP>(a, r, is_long, sq);
+    if constexpr (HINT) {
+        long_rows<T, OP>(a, r, is_long, sq);
+    } else {
+        if (longs) sq += long_rows_call<T, OP>(a, (int32_t)r, longs);
+    }
     if constexpr (OP == OP_RESID) {
         for (int off = 16; off > 0; off >>= 1) sq += __shfl_down_sync(0xffffffffu, sq, off);
         if ((tid & 31) == 0) sred[tid >> 5] = sq;
@@ -1335,7 +1395,8 @@ int keep_a_flag(int64_t n, int64_t nnz, int elem, int nvec, bool may_reserve,
     const double a_bytes = (double)nnz * (elem + 4) + 4.0 * (n + 1);
     const double bytes = a_bytes + (double)nvec * n * elem;
     const int rows = ((double)nnz > 5.5 * (double)n ? F_WIDE : 0) |
-                     ((double)nnz > LONG_AVG * (double)n ? F_LONG : 0);
+                     ((double)nnz > LONG_AVG * (double)n ? F_LONG : 0) |
+                     ((double)nnz > SPREAD_AVG * (double)n ? F_SPREAD : 0);
     if (!fits_l2(bytes, l2)) {
         // streaming: a chain holds the nonzeros of its leading rows in a
         // set-aside of kPartialL2 (shrinking a larger one that an L2-resident
@@ -1512,7 +1573,10 @@ int32_t launch_step(int op, const StepArgs<T>& a_in, cudaStream_t s) {
         if (op != OP_RESID) {
             const int rows_d = a_in.n <= sms * DIRECT_SMALL_ROWS ? DIRECT_SMALL_ROWS : DIRECT_L2_ROWS;
             cfg.blockDim = dim3(rows_d);
-            cfg.gridDim = dim3((unsigned)(((int64_t)a_in.n + rows_d - 1) / rows_d));
+            int64_t threads = a_in.n;
+            if (small && (a.flags & F_SPREAD))   // more warps for the same rows
+                threads = ((int64_t)a_in.n + SPREAD_ROWS - 1) / SPREAD_ROWS * 32;
+            cfg.gridDim = dim3((unsigned)((threads + rows_d - 1) / rows_d));
             // The next step is let in by a grid of at most LATE_MAX CTAs per SM only
             // when the previous one is done, by a larger one at once.  At once, the
             // CTAs of a third and fourth step come in too wherever there is room, to

@@ -91,3 +91,23 @@ def test_residual_with_long_rows(env, per_row):
     x, st = p.solve(big, b, m=1, tol=1e-30, x0=x0, max_cycles=1)
     r = b - p.spmv(big, x)
     assert abs(st["true_relres"] - float(r.norm() / b.norm())) <= 1e-13 * st["true_relres"]
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("n", [200, 1101, 1102, 1103, 32768])
+def test_few_rows_to_a_warp(env, n, dtype):
+    """More than 22 entries in the average row of a small system: four rows to a
+    warp, the last one with fewer, short and long."""
+    p, torch = env
+    tdt = torch.float64 if dtype == "f64" else torch.float32
+    lens = {r: 129 + r % 90 for r in range(0, n, 5)} if n < 5000 else {r: 400 for r in range(0, n, 16)}
+    A = dev_csr(p, torch, random_csr(n, 6, long_rows=lens, empty_rows={1}), dtype=tdt)
+    assert A.nnz > 22 * n
+    big = _streamed(p, torch, A, 5)
+    v = to_dev(torch, np.random.default_rng(9).standard_normal(A.n), tdt)
+    vb = torch.cat([v, torch.ones(big.n - A.n, dtype=tdt, device="cuda")])
+    assert p.chain_form(A, 7) == "direct" and p.chain_form(big, 7) == "staged"
+    assert torch.equal(p.spmv(big, vb)[: A.n], p.spmv(A, v))
+    R = p.Roots.from_complex(ROOTS)
+    assert torch.equal(p.apply_poly(big, R, vb)[: A.n], p.apply_poly(A, R, v))
+    assert torch.equal(p.apply_phi(big, R, vb)[: A.n], p.apply_phi(A, R, v))
