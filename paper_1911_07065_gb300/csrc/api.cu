@@ -148,7 +148,7 @@ static int32_t run_steps(const std::vector<Step>& plan, int i0, int i1, const in
     // limit cannot change)
     int32_t keep_rows = 0;
     const int keep = keep_a_flag(n, nnz, (int)sizeof(T), 3, reserve_l2, &keep_rows);
-    if (i0 == 0 && i1 == (int)plan.size() && chain_cluster_fits<T>(plan.size(), n, nnz)) {
+    if (i0 == 0 && i1 == (int)plan.size() && chain_cluster_fits<T>(plan.size(), n, nnz, s)) {
         PPG_TRY(launch_chain_cluster<T>(plan, rowptr, colind, vals, n, bufs, s));
         for (const Step& st : plan) bytes += step_bytes(st.op, st.flags, n, nnz, (int)sizeof(T));
         if (bytes_out) *bytes_out = bytes;
@@ -232,6 +232,15 @@ int device_sm_count() {
         if (dev >= 0) cached[dev].store(v, std::memory_order_relaxed);
     }
     return v;
+}
+
+bool stream_capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();   // (the legacy stream while another one is captured)
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
 }
 
 static int64_t pad_ld(int32_t n) { return ((int64_t)n + 63) / 64 * 64; }
@@ -620,8 +629,8 @@ static int32_t run_solve(SolveCore& c) {
     // (a chain that is one launch goes ahead whole: its result, basis column
     // j + 2, is not read by the update either)
     const bool whole = chain && !c.sweep &&
-                       (c.flex ? chain_cluster_fits<float>(chain->size(), n, nnz)
-                               : chain_cluster_fits<double>(chain->size(), n, nnz));
+                       (c.flex ? chain_cluster_fits<float>(chain->size(), n, nnz, s)
+                               : chain_cluster_fits<double>(chain->size(), n, nnz, s));
     const int nahead = whole ? (int)chain->size()
                        : (chain && !c.sweep)
                            ? std::max(0, std::min(kLookahead, (int)chain->size() - 1))
@@ -1217,8 +1226,8 @@ int32_t ppg_chain_form(const ppg_csr* A, int32_t steps, int32_t* form, void* str
     PPG_TRY(setup_device_pool());
     cudaStream_t s = (cudaStream_t)stream;
     const bool f64 = A->dtype == PPG_F64;
-    if (f64 ? chain_cluster_fits<double>((size_t)steps, A->n, A->nnz)
-            : chain_cluster_fits<float>((size_t)steps, A->n, A->nnz)) {
+    if (f64 ? chain_cluster_fits<double>((size_t)steps, A->n, A->nnz, s)
+            : chain_cluster_fits<float>((size_t)steps, A->n, A->nnz, s)) {
         *form = PPG_FORM_CLUSTER;
         return PPG_OK;
     }

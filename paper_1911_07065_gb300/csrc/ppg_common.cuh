@@ -238,6 +238,9 @@ struct DiagStore {
     ~DiagStore() { drop(); }
 };
 
+// whether work enqueued on `s` goes into a graph
+bool stream_capturing(cudaStream_t s);
+
 // algorithmic bytes of one fused step
 double step_bytes(int op, int flags, int64_t n, int64_t nnz, int elem);
 
@@ -273,7 +276,7 @@ int32_t run_plan(const std::vector<Step>& plan, const int32_t* rowptr,
 // A small system's whole chain in one launch (small_chain.cu): whether it takes
 // a plan of `steps` steps, and the plan's steps with the same buffers as run_plan's.
 template <typename T>
-bool chain_cluster_fits(size_t steps, int32_t n, int64_t nnz);
+bool chain_cluster_fits(size_t steps, int32_t n, int64_t nnz, cudaStream_t s);
 template <typename T>
 int32_t launch_chain_cluster(const std::vector<Step>& plan, const int32_t* rowptr,
                              const int32_t* colind, const T* vals, int32_t n, const Buffers& bufs,

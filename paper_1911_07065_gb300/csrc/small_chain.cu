@@ -73,7 +73,7 @@ __device__ __forceinline__ void cluster_wait() {
 }
 
 template <typename T, int R>
-__global__ void __launch_bounds__(CHAIN_THREADS)
+__global__ void __launch_bounds__(CHAIN_THREADS, 1)
 k_chain_cluster(const __grid_constant__ ChainArgs<T> a) {
     extern __shared__ __align__(16) unsigned char chain_x[];   // 2 x chunk of T
     T* const xs = reinterpret_cast<T*>(chain_x);
@@ -146,11 +146,20 @@ k_chain_cluster(const __grid_constant__ ChainArgs<T> a) {
                 if (e < most) {   // uniform: no FP64 issue for what no lane has
                     if (e < ordinary) acc = fma(v[i][e], x[e], acc);
                 }
-#pragma unroll 4
-            for (int e = CHAIN_E; e < ordinary; ++e) {
-                T xe;
-                ld_cluster(xe, at(__ldg(a.colind + k0[i] + e)) + cur);
-                acc = fma(__ldg(a.vals + k0[i] + e), xe, acc);
+            for (int e = CHAIN_E; e < ordinary; e += 4) {
+                // (past the end: the last entry again, so that the loads need no branch)
+                int32_t c[4];
+                T w[4], xe[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    c[u] = __ldg(a.colind + k0[i] + min(e + u, ordinary - 1));
+                    w[u] = __ldg(a.vals + k0[i] + min(e + u, ordinary - 1));
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) ld_cluster(xe[u], at(c[u]) + cur);
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (e + u < ordinary) acc = fma(w[u], xe[u], acc);
             }
             // rows of more than LONG_ROW entries, a warp for each
             for (unsigned todo = longs[i]; todo; todo &= todo - 1) {
@@ -274,19 +283,24 @@ bool cluster_possible() {
 
 }  // namespace
 
-// The line: FP64 where the cluster's multiply-adds (nnz + n a step) take less
-// than a step's launch (40 steps, launches against cluster: 2-D 50^2 87 / 40 us,
-// 100^2 86 / 79 us, 110^2 85 / 90 us; 3-D 20^3 86 / 79 us, 25^3 85 / 133 us), FP32
-// up to two rows a thread (50^2 83 / 21 us, 128^2 84 / 36 us).
+// The line, from 40 steps of p(A), launch by launch / in one cluster.  FP64: where
+// the cluster's multiply-adds (nnz + n a step) take less than a step's launch: 2-D
+// 50^2 79 / 43 us, 80^2 78 / 65, 90^2 78 / 77, 100^2 77 / 83; 3-D 18^3 78 / 64, 20^3
+// 79 / 79.  As a graph the launches cost less: 70^2 64 / 57, 80^2 64 / 68.  FP32: up
+// to two rows a thread (50^2 76 / 22, as a graph 45 / 26; 128^2 78 / 37 and 47 /
+// 40).  And at most CHAIN_E entries in the average row: what a row has beyond them is
+// read again in each step, with the chain of its gathers in the cluster's few warps
+// (FP64, 2,000 rows of 30: 160 / 236 us, 220 rows of 200: 620 / 2,330; FP32, 3,000
+// rows of 64: 248 / 460).
 template <typename T>
-bool chain_cluster_fits(size_t steps, int32_t n, int64_t nnz) {
-    if (n > CHAIN_CTAS * CHAIN_THREADS * CHAIN_ROWS) return false;
-    if (nnz + n > (sizeof(T) == 8 ? 64000 : 200000)) return false;
+bool chain_cluster_fits(size_t steps, int32_t n, int64_t nnz, cudaStream_t s) {
+    if (n > CHAIN_CTAS * CHAIN_THREADS * CHAIN_ROWS || nnz > (int64_t)CHAIN_E * n) return false;
+    if (sizeof(T) == 8 && nnz + n > 36000 && (nnz + n > 48000 || stream_capturing(s))) return false;
     if (steps < 2 || steps > (size_t)CHAIN_STEPS) return false;
     return cluster_possible<T>();
 }
-template bool chain_cluster_fits<double>(size_t, int32_t, int64_t);
-template bool chain_cluster_fits<float>(size_t, int32_t, int64_t);
+template bool chain_cluster_fits<double>(size_t, int32_t, int64_t, cudaStream_t);
+template bool chain_cluster_fits<float>(size_t, int32_t, int64_t, cudaStream_t);
 
 template <typename T>
 int32_t launch_chain_cluster(const std::vector<Step>& plan, const int32_t* rowptr,
