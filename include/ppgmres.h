@@ -196,7 +196,10 @@ int32_t ppg_build_poly(const ppg_csr* A, int32_t d, const double* v0,
  * limit of this process's context, never a device setting: when the matrix
  * and three vectors fit in 80 % of L2, a set-aside sized for the matrix,
  * which then stays resident across the roots; otherwise 48 MB, which holds
- * the nonzeros of the matrix's leading rows while the rest streams. */
+ * the nonzeros of the matrix's leading rows while the rest streams.  While
+ * `stream` is being captured into a graph the limit stays as it is.  (The first
+ * call of a process on a device loads the library's device code, which a
+ * capture does not allow: make one call before.) */
 int32_t ppg_apply_poly(const ppg_csr* A, const ppg_roots* r, const void* v,
                        void* y, void* stream);
 

@@ -143,17 +143,14 @@ static int32_t run_steps(const std::vector<Step>& plan, int i0, int i1, const in
         if (bytes_out) *bytes_out = 0.0;
         return PPG_OK;
     }
-    // (a small system reserves its share of L2 too, though its one launch makes no
-    // use of it: a larger one may come next inside a stream capture, where the
-    // limit cannot change)
-    int32_t keep_rows = 0;
-    const int keep = keep_a_flag(n, nnz, (int)sizeof(T), 3, reserve_l2, &keep_rows);
     if (i0 == 0 && i1 == (int)plan.size() && chain_cluster_fits<T>(plan.size(), n, nnz, s)) {
         PPG_TRY(launch_chain_cluster<T>(plan, rowptr, colind, vals, n, bufs, s));
         for (const Step& st : plan) bytes += step_bytes(st.op, st.flags, n, nnz, (int)sizeof(T));
         if (bytes_out) *bytes_out = bytes;
         return PPG_OK;
     }
+    int32_t keep_rows = 0;
+    const int keep = keep_a_flag(n, nnz, (int)sizeof(T), 3, s, reserve_l2, &keep_rows);
     const int sms = device_sm_count();
     for (int i = i0; i < i1; ++i) {
         const Step& st = plan[(size_t)i];
@@ -447,7 +444,7 @@ static int32_t build_core(const ppg_csr* A, int d, const double* v0, const ppg_o
             a.colind = A->colind;
             a.vals = (const double*)A->vals;
             a.n = n;
-            a.flags = keep_a_flag(a.n, A->nnz, 8, 3);
+            a.flags = keep_a_flag(a.n, A->nnz, 8, 3, s);
             a.x = vj;
             a.o0 = w;
             int32_t g = launch_step<double>(OP_SPMV, a, s);
@@ -575,7 +572,7 @@ static int32_t run_solve(SolveCore& c) {
         a.colind = c.A64->colind;
         a.vals = (const double*)c.A64->vals;
         a.n = n;
-        a.flags = keep_a_flag(a.n, c.A64->nnz, 8, 3);
+        a.flags = keep_a_flag(a.n, c.A64->nnz, 8, 3, s);
         if (c.opts.x0_given) {
             a.x = c.x;
             a.a0 = c.b;
@@ -686,7 +683,7 @@ static int32_t run_solve(SolveCore& c) {
         a.colind = c.A64->colind;
         a.vals = (const double*)c.A64->vals;
         a.n = n;
-        a.flags = keep_a_flag(a.n, c.A64->nnz, 8, 3);
+        a.flags = keep_a_flag(a.n, c.A64->nnz, 8, 3, s);
         a.o0 = w;
         if (c.flex) {
             float* zj = c.Z32 + (size_t)j * c.ldv;
@@ -786,7 +783,7 @@ static int32_t run_solve(SolveCore& c) {
         a.colind = c.A64->colind;
         a.vals = (const double*)c.A64->vals;
         a.n = n;
-        a.flags = keep_a_flag(a.n, c.A64->nnz, 8, 3);
+        a.flags = keep_a_flag(a.n, c.A64->nnz, 8, 3, s);
         a.x = c.x;
         a.a0 = c.b;
         a.o0 = c.V;
@@ -886,7 +883,7 @@ static int32_t run_solve_ext(SolveCore& c, const ppg_roots* inner, int rebuild_d
         a.colind = A->colind;
         a.vals = vals;
         a.n = n;
-        a.flags = keep_a_flag(n, nnz, 8, 3);
+        a.flags = keep_a_flag(n, nnz, 8, 3, s);
         a.x = xin;
         a.o0 = yout;
         const int32_t g = launch_step<double>(OP_SPMV, a, s);
@@ -1158,14 +1155,14 @@ int32_t ppg_spmv(const ppg_csr* A, const void* x, void* y, void* stream) {
         StepArgs<double> a{};
         a.rowptr = A->rowptr; a.colind = A->colind; a.vals = (const double*)A->vals; a.n = A->n;
         a.x = (const double*)x; a.o0 = (double*)y;
-        a.flags = keep_a_flag(A->n, A->nnz, 8, 2);
+        a.flags = keep_a_flag(A->n, A->nnz, 8, 2, s);
         int32_t g = launch_step<double>(OP_SPMV, a, s);
         return g < 0 ? g : PPG_OK;
     }
     StepArgs<float> a{};
     a.rowptr = A->rowptr; a.colind = A->colind; a.vals = (const float*)A->vals; a.n = A->n;
     a.x = (const float*)x; a.o0 = (float*)y;
-    a.flags = keep_a_flag(A->n, A->nnz, 4, 2);
+    a.flags = keep_a_flag(A->n, A->nnz, 4, 2, s);
     int32_t g = launch_step<float>(OP_SPMV, a, s);
     return g < 0 ? g : PPG_OK;
 }
@@ -1244,7 +1241,7 @@ int32_t ppg_chain_form(const ppg_csr* A, int32_t steps, int32_t* form, void* str
             }
         }
     }
-    const bool direct = A->n <= DIRECT_MAX_N || (keep_a_flag(A->n, A->nnz, f64 ? 8 : 4, 3) & F_KEEP_A);
+    const bool direct = A->n <= DIRECT_MAX_N || (keep_a_flag(A->n, A->nnz, f64 ? 8 : 4, 3, s) & F_KEEP_A);
     *form = direct ? PPG_FORM_DIRECT : PPG_FORM_STAGED;
     return PPG_OK;
 }
@@ -1425,7 +1422,7 @@ static int32_t stch_core(const ppg_csr* A, const ppg_roots* r, const double* b, 
     a.colind = A->colind;
     a.vals = vals;
     a.n = n;
-    a.flags = keep_a_flag(n, A->nnz, 8, 3);
+    a.flags = keep_a_flag(n, A->nnz, 8, 3, s);
     a.x = y;
     a.a0 = b;
     a.o0 = r1;

@@ -196,15 +196,16 @@ int32_t launch_ew_step(int op, const StepArgs<T>& a, const T* prodv, cudaStream_
 // F_KEEP_A when the matrix plus `nvec` work vectors fit comfortably in L2
 // (with F_WIDE where its rows are that long).
 // The first such request reserves an L2 set-aside for the matrix (a limit of
-// the process's context on the current device); with may_reserve = false
+// the process's context on the current device; not while `s` is being captured,
+// which a change of the limit would invalidate); with may_reserve = false
 // nothing is reserved and F_KEEP_A is returned only if a set-aside large
 // enough already exists on this device.
 // keep_rows (root-step chains only): for a matrix that does not fit, the
 // number of leading rows whose nonzeros a chain holds in an L2 set-aside of
-// about 48 MB, which is set to that size (with may_reserve; otherwise the
-// set-aside in place, if any, is used); 0 without a set-aside.  Other callers
+// about 48 MB, which is set to that size (with may_reserve and outside a capture;
+// otherwise the set-aside in place, if any, is used); 0 without a set-aside.  Other callers
 // pass nullptr and leave the set-aside as it is.
-int keep_a_flag(int64_t n, int64_t nnz, int elem, int nvec, bool may_reserve = true,
+int keep_a_flag(int64_t n, int64_t nnz, int elem, int nvec, cudaStream_t s, bool may_reserve = true,
                 int32_t* keep_rows = nullptr);
 
 // at least the partial sums any residual step of n rows writes (one per CTA)

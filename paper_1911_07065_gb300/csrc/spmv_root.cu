@@ -1318,9 +1318,9 @@ static int current_device() {
     return dev;
 }
 
-static size_t reserve_l2_for(int dev, size_t bytes) {
+static size_t reserve_l2_for(int dev, size_t bytes, cudaStream_t s) {
     const size_t have = g_l2_reserved[dev].load(std::memory_order_relaxed);
-    if (bytes <= have) return have;
+    if (bytes <= have || stream_capturing(s)) return have;
     int maxp = 0;
     if (cudaDeviceGetAttribute(&maxp, cudaDevAttrMaxPersistingL2CacheSize, dev) != cudaSuccess ||
         maxp <= 0) {
@@ -1341,9 +1341,9 @@ static size_t reserve_l2_for(int dev, size_t bytes) {
 // Set the set-aside to `bytes` exactly (shrinking or growing it; persisting
 // lines back to normal first).  Returns the set-aside now in place (the
 // driver rounds the request to its granularity).
-static size_t set_l2_exact(int dev, size_t bytes) {
+static size_t set_l2_exact(int dev, size_t bytes, cudaStream_t s) {
     const size_t have = g_l2_reserved[dev].load(std::memory_order_relaxed);
-    if (g_l2_asked[dev].load(std::memory_order_relaxed) == bytes) return have;
+    if (g_l2_asked[dev].load(std::memory_order_relaxed) == bytes || stream_capturing(s)) return have;
     int maxp = 0;
     if (cudaDeviceGetAttribute(&maxp, cudaDevAttrMaxPersistingL2CacheSize, dev) != cudaSuccess ||
         maxp <= 0) {
@@ -1385,7 +1385,7 @@ static int l2_bytes(int dev) {
 // a chain's matrix and vectors fit comfortably in L2
 static bool fits_l2(double bytes, int l2) { return bytes <= 0.8 * (double)l2; }
 
-int keep_a_flag(int64_t n, int64_t nnz, int elem, int nvec, bool may_reserve,
+int keep_a_flag(int64_t n, int64_t nnz, int elem, int nvec, cudaStream_t s, bool may_reserve,
                 int32_t* keep_rows) {
     if (keep_rows) *keep_rows = 0;
     const int dev = current_device();
@@ -1403,7 +1403,7 @@ int keep_a_flag(int64_t n, int64_t nnz, int elem, int nvec, bool may_reserve,
         // workload left: an unused 76 MB set-aside cost the 160^3 FP32 chains
         // 11 %), and streams the rest
         if (!keep_rows) return rows;
-        const size_t have = may_reserve ? set_l2_exact(dev, kPartialL2)
+        const size_t have = may_reserve ? set_l2_exact(dev, kPartialL2, s)
                                         : g_l2_reserved[dev].load(std::memory_order_relaxed);
         const double held = 0.9 * (double)have / (a_bytes / (double)n);
         *keep_rows = (int32_t)(held < (double)n ? held : (double)n);
@@ -1411,7 +1411,7 @@ int keep_a_flag(int64_t n, int64_t nnz, int elem, int nvec, bool may_reserve,
     }
     const size_t need = (size_t)(a_bytes * 1.05);
     if (may_reserve) {
-        reserve_l2_for(dev, need);
+        reserve_l2_for(dev, need, s);
         return F_KEEP_A | rows;
     }
     // no change to the context: the hint only where a set-aside exists
