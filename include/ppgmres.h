@@ -120,8 +120,11 @@ typedef struct ppg_stats {
     /* filled when opts.timing = 1: the fused SpMV-root kernels of the
      * polynomial chains (Algorithms 1 and 3) */
     double  poly_ms;        /* summed CUDA-event time of those launches */
-    int64_t poly_launches;
-    double  poly_bytes;     /* algorithmic bytes of those launches */
+    int64_t poly_launches;  /* a chain in one launch (PPG_FORM_CLUSTER) counts as one */
+    double  poly_bytes;     /* algorithmic bytes of those launches, in the form they read the
+                               matrix in: PPG_FORM_CLUSTER the CSR once a chain,
+                               PPG_FORM_DIAGONALS a mask and the values that are not one
+                               throughout their diagonal */
     double  ortho_ms;       /* CGS2 + Givens kernels */
 } ppg_stats;
 

@@ -145,8 +145,7 @@ static int32_t run_steps(const std::vector<Step>& plan, int i0, int i1, const in
     }
     if (i0 == 0 && i1 == (int)plan.size() && chain_cluster_fits<T>(plan.size(), n, nnz, s)) {
         PPG_TRY(launch_chain_cluster<T>(plan, rowptr, colind, vals, n, bufs, s));
-        for (const Step& st : plan) bytes += step_bytes(st.op, st.flags, n, nnz, (int)sizeof(T));
-        if (bytes_out) *bytes_out = bytes;
+        if (bytes_out) *bytes_out = chain_cluster_bytes(plan, n, nnz, (int)sizeof(T));
         return PPG_OK;
     }
     int32_t keep_rows = 0;
@@ -183,6 +182,7 @@ static int32_t run_steps(const std::vector<Step>& plan, int i0, int i1, const in
         int32_t rc = launch_step<T>(st.op, a, s);
         if (rc < 0) return rc;
         bytes += step_bytes(st.op, st.flags, n, nnz, (int)sizeof(T));
+        if (diag) bytes += diag->bytes_beyond_csr(n, nnz);
     }
     if (bytes_out) *bytes_out = bytes;
     return PPG_OK;
@@ -670,9 +670,14 @@ static int32_t run_solve(SolveCore& c) {
             PPG_TRY(launch_cast_f64_f32(c.V + (size_t)j * c.ldv, c.v32, n, s));
         }
         ev_poly[e].start(s);
-        if (chain && upto > 0) PPG_TRY(chain_steps(j, 0, upto, by));
+        if (chain && upto > 0) {
+            PPG_TRY(chain_steps(j, 0, upto, by));
+            if (upto == (int)chain->size()) ev_poly[e].stop(s);
+        }
         return PPG_OK;
     };
+    const int64_t p_launches = pp && chain_cluster_fits<double>(c.p_plan.size(), n, nnz, s)
+                                   ? 1 : (int64_t)c.p_plan.size();   // (FP64: the restart's)
     // the rest of step j from chain step `from` on
     bool scaled = false;   // basis column j + 1 has its scale
     auto finish_step = [&](int j, int e, int from, double* by) -> int32_t {
@@ -687,24 +692,27 @@ static int32_t run_solve(SolveCore& c) {
         a.o0 = w;
         if (c.flex) {
             float* zj = c.Z32 + (size_t)j * c.ldv;
-            if (pp) {
+            if (pp && from < (int)chain->size()) {
                 double b2 = 0;
                 PPG_TRY(chain_steps(j, from, (int)chain->size(), &b2));
                 *by += b2;
-            } else {
+                ev_poly[e].stop(s);
+            } else if (!pp) {
                 PPG_CUDA(cudaMemcpyAsync(zj, c.v32, sizeof(float) * n, cudaMemcpyDeviceToDevice,
                                          s));
+                ev_poly[e].stop(s);
             }
-            ev_poly[e].stop(s);
             PPG_TRY(launch_cast_f32_f64(zj, c.u, n, s));
             a.x = c.u;
             const int32_t g = launch_step<double>(OP_SPMV, a, s);
             if (g < 0) return g;
         } else if (pp) {
-            double b2 = 0;
-            PPG_TRY(chain_steps(j, from, (int)chain->size(), &b2));
-            *by += b2;
-            ev_poly[e].stop(s);
+            if (from < (int)chain->size()) {
+                double b2 = 0;
+                PPG_TRY(chain_steps(j, from, (int)chain->size(), &b2));
+                *by += b2;
+                ev_poly[e].stop(s);
+            }
         } else {
             a.x = vj;
             const int32_t g = launch_step<double>(OP_SPMV, a, s);
@@ -744,6 +752,7 @@ static int32_t run_solve(SolveCore& c) {
             c.st.ortho_ms += ev_orth[e].ms();
             c.st.poly_bytes += by_step;
             c.st.poly_launches += chain ? (c.sweep ? sweep_chain_launches(c.sweep, *chain)
+                                           : whole ? 1
                                                    : (int64_t)chain->size())
                                         : (c.flex ? 0 : 1);
             c.st.mvps += pp ? d : 1;   // flexible form: d-1 in p(A) v_j, one for A z_j
@@ -772,7 +781,7 @@ static int32_t run_solve(SolveCore& c) {
                                      (const double*)c.A64->vals, n, nnz, pb, s, &by));
             ev_restart.stop(s);
             c.st.poly_bytes += by;
-            c.st.poly_launches += (int64_t)c.p_plan.size();
+            c.st.poly_launches += p_launches;
             c.st.mvps += d - 1;
         } else {
             PPG_TRY(launch_gemv_acc<double>(c.V, c.ldv, k, c.gs.y, c.x, n, true, s));

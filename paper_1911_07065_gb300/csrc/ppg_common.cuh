@@ -229,8 +229,13 @@ struct DiagStore {
         fresh = false;
     }
     // Wait for the search; without a form the memory goes back and the steps are
-    // the kernels that know of none.  `pinned`: room for an int32_t.
+    // the kernels that know of none.  `pinned`: room for three int32_t.
     int32_t settle(void* pinned);
+    int own = 0;   // (settled) diagonals with values of their own
+    // algorithmic bytes of a settled step less those of the CSR step
+    double bytes_beyond_csr(int64_t n, int64_t nnz) const {
+        return f.head ? (4.0 * own + f.mask_bytes) * (double)n - 8.0 * (double)nnz - 4.0 * (double)(n + 1) : 0.0;
+    }
     void drop() {
         if (mem) cudaFreeAsync(mem, s);
         mem = nullptr;
@@ -282,6 +287,8 @@ template <typename T>
 int32_t launch_chain_cluster(const std::vector<Step>& plan, const int32_t* rowptr,
                              const int32_t* colind, const T* vals, int32_t n, const Buffers& bufs,
                              cudaStream_t s);
+// what that launch has to move: the matrix once, the chain's vectors in and out
+double chain_cluster_bytes(const std::vector<Step>& plan, int64_t n, int64_t nnz, int elem);
 
 // ---------------------------------------------------------------------------
 // Multi-root fused sweep (sweep.cu): Algorithm 3 on a plan's reordered FP32

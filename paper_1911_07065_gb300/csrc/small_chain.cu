@@ -302,6 +302,13 @@ bool chain_cluster_fits(size_t steps, int32_t n, int64_t nnz, cudaStream_t s) {
 template bool chain_cluster_fits<double>(size_t, int32_t, int64_t, cudaStream_t);
 template bool chain_cluster_fits<float>(size_t, int32_t, int64_t, cudaStream_t);
 
+double chain_cluster_bytes(const std::vector<Step>& plan, int64_t n, int64_t nnz, int elem) {
+    const Step& head = plan[0];
+    const bool phi = head.op == OP_PHI_REAL || head.op == OP_SPMV;
+    const int vec = !phi && !(head.flags & F_PZERO) ? 3 : 2;   // in, out (read too where it adds to it)
+    return (double)nnz * (elem + 4) + 4.0 * (double)(n + 1) + (double)vec * elem * (double)n;
+}
+
 template <typename T>
 int32_t launch_chain_cluster(const std::vector<Step>& plan, const int32_t* rowptr,
                              const int32_t* colind, const T* vals, int32_t n, const Buffers& bufs,

@@ -1496,9 +1496,12 @@ int32_t DiagStore::build(const int32_t* rowptr, const int32_t* colind, const flo
 
 int32_t DiagStore::settle(void* pinned) {
     if (!f.head) return PPG_OK;
-    PPG_CUDA(cudaMemcpyAsync(pinned, f.head, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    PPG_CUDA(cudaMemcpyAsync(pinned, f.head, 3 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     PPG_CUDA(cudaStreamSynchronize(s));
-    if (*(const int32_t*)pinned != 0) drop();
+    const int32_t* head = (const int32_t*)pinned;
+    own = head[1];
+    for (uint32_t one = (uint32_t)head[2]; one; one &= one - 1) --own;
+    if (head[0] != 0) drop();
     return PPG_OK;
 }
 

@@ -104,3 +104,34 @@ def test_launches_of_a_small_system(env):
     before = p.lib.ppg_launch_count()
     p.build_poly(A, 20, v)
     assert p.lib.ppg_launch_count() - before <= 2 * 20 + 12
+
+
+def test_chain_statistics_of_a_small_system(env):
+    """A chain in one launch counts as one, with the matrix read once."""
+    p, torch = env
+    H = synth.cd2d(50, 0.5)
+    A = dev_csr(p, torch, H)
+    b = to_dev(torch, np.random.default_rng(1).standard_normal(A.n))
+    R = p.build_poly(A, 10, b)
+    _, st = p.solve(A, b, m=20, tol=1e-8, roots=R, timing=True)
+    chains = st["iters"] + st["cycles"]
+    assert st["poly_launches"] == chains and st["poly_launches"] < st["launches"]
+    csr = 12 * H.rowptr[-1] + 4 * (H.n + 1)
+    assert st["poly_bytes"] == st["iters"] * (csr + 16 * H.n) + st["cycles"] * (csr + 24 * H.n)
+    assert 0 < st["poly_ms"]
+
+
+def test_chain_statistics_by_diagonals(env):
+    """A grid's FP32 steps by its diagonals, all of one value: a byte of mask to a row
+    and two to four vectors; and by the CSR without the form."""
+    p, torch = env
+    for name, kw in (("grid", CASES["one_value_each"]), ("none", CASES["forty"])):
+        H = _banded(**kw)
+        A = dev_csr(p, torch, H)
+        b = to_dev(torch, np.random.default_rng(1).standard_normal(A.n))
+        R = p.Roots.from_complex(_roots())
+        _, st = p.solve_flex(A, A.astype(torch.float32), b, R, m=2, tol=1e-30, max_cycles=1, timing=True)
+        per_row = st["poly_bytes"] / st["poly_launches"] / A.n
+        csr = 8 * H.rowptr[-1] / H.n
+        assert (1 + 8 <= per_row <= 1 + 16) if name == "grid" else (csr + 8 <= per_row <= csr + 4 + 16.1)
+        assert st["poly_launches"] == 2 * 33
