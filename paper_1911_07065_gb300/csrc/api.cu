@@ -143,8 +143,8 @@ static int32_t run_steps(const std::vector<Step>& plan, int i0, int i1, const in
         if (bytes_out) *bytes_out = 0.0;
         return PPG_OK;
     }
-    if (i0 == 0 && i1 == (int)plan.size() && chain_cluster_fits<T>(plan.size(), n, nnz, s)) {
-        PPG_TRY(launch_chain_cluster<T>(plan, rowptr, colind, vals, n, bufs, s));
+    if (i0 == 0 && i1 == (int)plan.size() && chain_cluster_fits<T>(plan.size(), n, nnz, s) &&
+        launch_chain_cluster<T>(plan, rowptr, colind, vals, n, bufs, s)) {
         if (bytes_out) *bytes_out = chain_cluster_bytes(plan, n, nnz, (int)sizeof(T));
         return PPG_OK;
     }
@@ -370,8 +370,9 @@ static int32_t orthogonalise(SolveCore& c, int ldh, int j, double* w, bool with_
     *scaled = !c.opts.cgs2_fused && arnoldi_small_fits(c.A64->n, j + 1);
     if (*scaled) {
         if (ev) ev->start(c.s);
-        return launch_arnoldi_small(c.V, c.ldv, j, w, c.A64->n, with_self, c.gs, ldh, givens, bnorm, brtol,
-                                    c.s);
+        *scaled = launch_arnoldi_small(c.V, c.ldv, j, w, c.A64->n, with_self, c.gs, ldh, givens, bnorm, brtol,
+                                       c.s);
+        if (*scaled) return PPG_OK;
     }
     PPG_TRY(cgs2_column(c, j, w, with_self, ev));
     return launch_finish_column(c.gs, ldh, j, c.ows.h1, c.ows.h2, c.ows.nrm, givens, bnorm, brtol, c.s);

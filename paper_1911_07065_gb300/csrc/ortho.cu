@@ -1211,7 +1211,7 @@ __global__ void __launch_bounds__(SMALL_THREADS + 32, 1) k_arnoldi_small(const S
     cluster_wait();
 }
 
-static int32_t small_launch(const SmallArnoldi& a, size_t smem, bool probe, int* clusters, cudaStream_t s) {
+static bool small_launch(const SmallArnoldi& a, size_t smem, bool probe, int* clusters, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(SMALL_CTAS);
     cfg.blockDim = dim3(SMALL_THREADS + 32);
@@ -1235,16 +1235,14 @@ static int32_t small_launch(const SmallArnoldi& a, size_t smem, bool probe, int*
             cudaGetLastError();
             *clusters = 0;
         }
-        return PPG_OK;
+        return true;
     }
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_arnoldi_small, a);
+    if (cudaLaunchKernelEx(&cfg, k_arnoldi_small, a) != cudaSuccess) {
+        cudaGetLastError();   // (fewer SMs at hand than when the device was asked)
+        return false;
+    }
     ++g_launches;
-    if (e != cudaSuccess) {
-        set_cuda_error(e, "cudaLaunchKernelEx(k_arnoldi_small)");
-        cudaGetLastError();
-        return PPG_ERR_CUDA;
-    }
-    return PPG_OK;
+    return true;
 }
 
 // Up to 300,000 basis entries (and a CTA's rows of w and one column in shared
@@ -1268,7 +1266,7 @@ bool arnoldi_small_fits(int32_t n, int ncol) {
     return k > 0;
 }
 
-int32_t launch_arnoldi_small(const double* V, int64_t ldv, int j, double* w, int32_t n, bool with_self,
+bool launch_arnoldi_small(const double* V, int64_t ldv, int j, double* w, int32_t n, bool with_self,
                              const GmresState& st, int ldh, bool givens, double bnorm, double brtol,
                              cudaStream_t s) {
     SmallArnoldi a{};

@@ -280,11 +280,12 @@ int32_t run_plan(const std::vector<Step>& plan, const int32_t* rowptr,
                  bool reserve_l2 = true, DiagStore* diag = nullptr);
 
 // A small system's whole chain in one launch (small_chain.cu): whether it takes
-// a plan of `steps` steps, and the plan's steps with the same buffers as run_plan's.
+// a plan of `steps` steps, and the plan's steps with the same buffers as run_plan's
+// (false: the launch was refused, and nothing is enqueued).
 template <typename T>
 bool chain_cluster_fits(size_t steps, int32_t n, int64_t nnz, cudaStream_t s);
 template <typename T>
-int32_t launch_chain_cluster(const std::vector<Step>& plan, const int32_t* rowptr,
+bool launch_chain_cluster(const std::vector<Step>& plan, const int32_t* rowptr,
                              const int32_t* colind, const T* vals, int32_t n, const Buffers& bufs,
                              cudaStream_t s);
 // what that launch has to move: the matrix once, the chain's vectors in and out
@@ -365,8 +366,9 @@ int32_t launch_finish_column(const GmresState& st, int ldh, int j,
                              double breakdown_rtol, cudaStream_t s);
 // CGS2 of basis column j + 1 (w) against columns 0..j, launch_finish_column and
 // the scaling of w by 1 / h_{j+1,j} in one launch, for a system small enough
+// (false: the launch was refused, and nothing is enqueued)
 bool arnoldi_small_fits(int32_t n, int ncol);
-int32_t launch_arnoldi_small(const double* V, int64_t ldv, int j, double* w, int32_t n, bool with_self,
+bool launch_arnoldi_small(const double* V, int64_t ldv, int j, double* w, int32_t n, bool with_self,
                              const GmresState& st, int ldh, bool givens, double bnorm, double brtol,
                              cudaStream_t s);
 int32_t launch_scale(const double* x, double* y, int32_t n, const double* scal_ptr,

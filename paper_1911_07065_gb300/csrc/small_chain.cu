@@ -310,7 +310,7 @@ double chain_cluster_bytes(const std::vector<Step>& plan, int64_t n, int64_t nnz
 }
 
 template <typename T>
-int32_t launch_chain_cluster(const std::vector<Step>& plan, const int32_t* rowptr,
+bool launch_chain_cluster(const std::vector<Step>& plan, const int32_t* rowptr,
                              const int32_t* colind, const T* vals, int32_t n, const Buffers& bufs,
                              cudaStream_t s) {
     ChainArgs<T> a;
@@ -335,18 +335,17 @@ int32_t launch_chain_cluster(const std::vector<Step>& plan, const int32_t* rowpt
         e = launch_cluster<T, 1>(a, a.chunk, smem, false, nullptr, s);
     else
         e = launch_cluster<T, 2>(a, (a.chunk / 2 + 31) / 32 * 32, smem, false, nullptr, s);
-    ++g_launches;
-    if (e != cudaSuccess) {
-        set_cuda_error(e, "cudaLaunchKernelEx(k_chain_cluster)");
+    if (e != cudaSuccess) {   // (fewer SMs at hand than when the device was asked)
         cudaGetLastError();
-        return PPG_ERR_CUDA;
+        return false;
     }
-    return PPG_OK;
+    ++g_launches;
+    return true;
 }
-template int32_t launch_chain_cluster<double>(const std::vector<Step>&, const int32_t*,
+template bool launch_chain_cluster<double>(const std::vector<Step>&, const int32_t*,
                                               const int32_t*, const double*, int32_t,
                                               const Buffers&, cudaStream_t);
-template int32_t launch_chain_cluster<float>(const std::vector<Step>&, const int32_t*,
+template bool launch_chain_cluster<float>(const std::vector<Step>&, const int32_t*,
                                              const int32_t*, const float*, int32_t, const Buffers&,
                                              cudaStream_t);
 
