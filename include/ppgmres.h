@@ -18,8 +18,14 @@
  *    the host (build_poly, solve, stability_check, csr_validate)
  *    synchronise the stream before returning; apply_poly, apply_phi, spmv,
  *    csr_transpose and adjoint_vals_grad are asynchronous.
- *  - Scratch memory is taken stream-ordered (cudaMallocAsync) and returned
- *    (cudaFreeAsync) before the call returns.
+ *  - Scratch memory is taken stream-ordered (cudaMallocAsync) from the device's
+ *    default pool and returned (cudaFreeAsync) before the call returns; the pool
+ *    keeps it for later calls.  Beside its work vectors, an FP32 chain of 20 or
+ *    more root steps over a matrix larger than L2 (apply_poly, apply_phi,
+ *    solve_flex) tries to take room for the matrix by its diagonals: at most 4 n
+ *    (2 nnz / n + 1.5) bytes, twice the matrix's values, and only out of what
+ *    the pool holds or if it is at most an eighth of the device's free memory (in
+ *    a capture, as part of the graph's memory).  Without it the same steps run on the CSR, with the same results.
  *  - Return codes: 0 = success, > 0 = soft status, < 0 = error (see
  *    PPG_* below; ppg_strerror gives a message).  No C++ exception crosses
  *    this interface.  After PPG_ERR_CUDA the CUDA error is also reported by

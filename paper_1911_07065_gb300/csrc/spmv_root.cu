@@ -1454,6 +1454,24 @@ static int step_resident_ctas() {
 // (1.2e6 rows of seven random entries, 60 steps: 0.76 -> 1.07 ms).
 constexpr int64_t DIAG_MIN_STEPS = 20;
 
+// Scratch that a call can do without: out of what the pool holds, or at most an
+// eighth of the device's free memory, since the pool keeps what it has once taken
+// and another allocator's next request would go without.  (In a capture the memory
+// is the graph's, and the device must not be asked.)
+static bool scratch_at_hand(int dev, size_t need, cudaStream_t s) {
+    if (stream_capturing(s)) return true;
+    cudaMemPool_t pool;
+    uint64_t held = 0, used = 0;
+    size_t free_bytes = 0, total = 0;
+    const bool ok = cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess &&
+                    cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
+                    cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess &&
+                    (held - used >= need ||
+                     (cudaMemGetInfo(&free_bytes, &total) == cudaSuccess && need <= free_bytes / 8));
+    cudaGetLastError();
+    return ok;
+}
+
 int32_t DiagStore::build(const int32_t* rowptr, const int32_t* colind, const float* vals, int32_t n,
                          int64_t nnz, int64_t steps, cudaStream_t stream) {
     if (n <= DIRECT_MAX_N || n > (1 << 30) || steps < DIAG_MIN_STEPS || nnz < n) return PPG_OK;
@@ -1466,7 +1484,8 @@ int32_t DiagStore::build(const int32_t* rowptr, const int32_t* colind, const flo
     const int32_t ld = (n + DIAG_PAD - 1) / DIAG_PAD * DIAG_PAD;
     f.mask_bytes = most <= 8 ? 1 : most <= 16 ? 2 : 4;
     const size_t b_vals = (size_t)most * ld * sizeof(float);
-    if (cudaMallocAsync(&mem, 1024 + b_vals + (size_t)ld * f.mask_bytes, stream) != cudaSuccess) {
+    const size_t need = 1024 + b_vals + (size_t)ld * f.mask_bytes;
+    if (!scratch_at_hand(dev, need, stream) || cudaMallocAsync(&mem, need, stream) != cudaSuccess) {
         cudaGetLastError();   // the CSR steps need none of it
         mem = nullptr;
         return PPG_OK;

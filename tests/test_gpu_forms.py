@@ -1,5 +1,9 @@
 """GPU: the forms of a chain and of an Arnoldi step are the ones taken.  Each
 has another to fall back on with the same results, so results do not show it."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -135,3 +139,30 @@ def test_chain_statistics_by_diagonals(env):
         csr = 8 * H.rowptr[-1] / H.n
         assert (1 + 8 <= per_row <= 1 + 16) if name == "grid" else (csr + 8 <= per_row <= csr + 4 + 16.1)
         assert st["poly_launches"] == 2 * 33
+
+
+def test_no_room_for_the_diagonal_form(env):
+    """In a process of its own, whose other allocator holds all but 1.5 GB: the form's
+    250 MB stay untaken, and the result is that of the CSR steps."""
+    code = """
+import sys
+sys.path.insert(0, "tests")
+import numpy as np, torch, paper_1911_07065_gb300 as p
+from test_gpu_diagonals import GRID, _banded, _roots
+H = _banded(GRID, n=5_000_000)
+A = p.CSR.from_host(H.rowptr, H.colind, H.vals, dtype=torch.float32)
+v = torch.ones(A.n, dtype=torch.float32, device="cuda")
+R = p.Roots.from_complex(_roots())
+torch.cuda.synchronize()
+held = torch.empty(torch.cuda.mem_get_info()[0] - 1500 * 2**20, dtype=torch.uint8, device="cuda")
+assert p.chain_form(A, 33) == "staged"
+y = p.apply_poly(A, R, v)
+torch.cuda.synchronize()
+assert torch.cuda.mem_get_info()[0] > 1300 * 2**20
+del held
+torch.cuda.empty_cache()
+assert p.chain_form(A, 33) == "diagonals"
+assert torch.equal(p.apply_poly(A, R, v), y)
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=root, timeout=300)
