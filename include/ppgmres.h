@@ -398,8 +398,9 @@ int32_t ppg_build_poly_checked(const ppg_csr* A, int32_t d, const double* v0,
  *              NULL: rows are grouped by breadth-first growth over the
  *              pattern of A from the lowest-numbered row not yet placed
  *   tile_rows  rows per tile, a multiple of 32 in [32, 16384]
- *   fuse       1: fuse pairs when the halos total at most 60 % of n and a
- *              tile fits in shared memory; 0: never (the plain chain on the
+ *   fuse       1: fuse pairs when the halos total at most 60 % of n, a tile
+ *              fits in shared memory and no row has more than 128 entries
+ *              (such rows are a warp's work in the plain chain); 0: never (the plain chain on the
  *              reordered matrix, for comparison)
  * The plan owns device memory (cudaMalloc, about the size of A plus 8n
  * bytes) until ppg_sweep_plan_destroy.  Synchronises `stream`.  Errors:

@@ -193,8 +193,11 @@ int32_t launch_step(int op, const StepArgs<T>& a, cudaStream_t s);
 template <typename T>
 int32_t launch_ew_step(int op, const StepArgs<T>& a, const T* prodv, cudaStream_t s);
 
-// F_KEEP_A when the matrix plus `nvec` work vectors fit comfortably in L2
-// (with F_WIDE where its rows are that long).
+// F_WIDE, F_LONG and F_SPREAD as the matrix's rows are
+int row_flags(int64_t n, int64_t nnz);
+
+// F_KEEP_A when the matrix plus `nvec` work vectors fit comfortably in L2, with
+// row_flags.
 // The first such request reserves an L2 set-aside for the matrix (a limit of
 // the process's context on the current device; not while `s` is being captured,
 // which a change of the limit would invalidate); with may_reserve = false

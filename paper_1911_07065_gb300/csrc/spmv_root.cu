@@ -1,9 +1,9 @@
 // Fused CSR SpMV + root update: one pass over A per root of the GMRES
 // polynomial (Algorithm 1: phi(A) v, Algorithm 3: p(A) v), plus the plain
-// SpMV and the residual b - A x.  Two kernels with the same arithmetic
-// (each row summed in stored order, one fused multiply-add per nonzero,
-// acc = fma(val, x[col], acc), then the same epilogue), so their results
-// are bit-identical:
+// SpMV and the residual b - A x.  Two kernels with the same arithmetic (one fused
+// multiply-add per nonzero, acc = fma(val, x[col], acc); a row of up to LONG_ROW
+// entries summed in stored order, a longer one by a warp, long_rows; then the same
+// epilogue), so their results are bit-identical:
 //
 // k_spmv_step, for a matrix streamed from HBM: a CTA owns a tile of rows
 // (256 in FP64, 512 in FP32: two per thread).  It copies the tile's column
@@ -962,19 +962,19 @@ k_spmv_step(const StepArgs<T> a) {
     // now; everything up to griddepcontrol.wait reads only the matrix, which
     // no step writes, so it overlaps the previous step's tail.
     asm volatile("griddepcontrol.launch_dependents;");
+    static_assert(!DG || OP != OP_RESID, "residuals take the matrix in FP64");
     if constexpr (DG) {
         if (__ldg(a.diag.head) == 0) {   // uniform over the grid
             __shared__ __align__(16) DiagSlot slot[DIAG_MAX];
             __shared__ uint64_t bar;
             double sq = 0.0;
             int halves = 1, rows = nrows;
-            if (OP != OP_RESID && __ldg(a.diag.head + 3)) {   // two tiles on every other CTA
+            if (__ldg(a.diag.head + 3)) {   // two tiles on every other CTA
                 if (blockIdx.x & 1) return;
                 halves = (int64_t)a.n - row0 > ROWS ? 2 : 1;
                 rows = (int)min((int64_t)a.n - row0, (int64_t)2 * ROWS);
             }
             diag_tile<T, OP, NT, RPT>(a, (int32_t)row0, rows, (float*)stage, slot, &bar, sq, halves);
-            if constexpr (OP == OP_RESID) block_sq<NT>(sq, sred, a.part);
             return;
         }
     }
@@ -1120,9 +1120,8 @@ k_spmv_step(const StepArgs<T> a) {
 // Direct-read step: the same step, one row per thread, the row's matrix
 // entries read straight into registers (up to PRE of them) before the wait
 // on the previous step -- no shared-memory staging round, so the latency
-// chain of a step is row pointers -> (wait) -> gathers -> epilogue.  Each
-// row is summed in stored order with one FMA per nonzero and the same
-// epilogue as k_spmv_step: bit-identical results.  Two uses:
+// chain of a step is row pointers -> (wait) -> gathers -> epilogue.  The
+// sums and the epilogue are k_spmv_step's: bit-identical results.  Two uses:
 // * small systems (PRE = 8, no register bound): a step is a handful of CTAs,
 //   and latency, not bytes, sets its time;
 // * a matrix held in L2 (F_KEEP_A; the preloads carry the evict-last hint):
@@ -1385,6 +1384,11 @@ static int l2_bytes(int dev) {
 // a chain's matrix and vectors fit comfortably in L2
 static bool fits_l2(double bytes, int l2) { return bytes <= 0.8 * (double)l2; }
 
+int row_flags(int64_t n, int64_t nnz) {
+    return ((double)nnz > 5.5 * (double)n ? F_WIDE : 0) | ((double)nnz > LONG_AVG * (double)n ? F_LONG : 0) |
+           ((double)nnz > SPREAD_AVG * (double)n ? F_SPREAD : 0);
+}
+
 int keep_a_flag(int64_t n, int64_t nnz, int elem, int nvec, cudaStream_t s, bool may_reserve,
                 int32_t* keep_rows) {
     if (keep_rows) *keep_rows = 0;
@@ -1394,9 +1398,7 @@ int keep_a_flag(int64_t n, int64_t nnz, int elem, int nvec, cudaStream_t s, bool
     if (l2 <= 0 || n <= 0) return 0;
     const double a_bytes = (double)nnz * (elem + 4) + 4.0 * (n + 1);
     const double bytes = a_bytes + (double)nvec * n * elem;
-    const int rows = ((double)nnz > 5.5 * (double)n ? F_WIDE : 0) |
-                     ((double)nnz > LONG_AVG * (double)n ? F_LONG : 0) |
-                     ((double)nnz > SPREAD_AVG * (double)n ? F_SPREAD : 0);
+    const int rows = row_flags(n, nnz);
     if (!fits_l2(bytes, l2)) {
         // streaming: a chain holds the nonzeros of its leading rows in a
         // set-aside of kPartialL2 (shrinking a larger one that an L2-resident
@@ -1542,7 +1544,9 @@ template <typename T, bool DG, bool LR>
 static cudaError_t launch_op(cudaLaunchConfig_t& cfg, int op, const StepArgs<T>& a) {
     switch (op) {
         case OP_SPMV: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_SPMV, DG, LR>, a);
-        case OP_RESID: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_RESID, DG, LR>, a);
+        case OP_RESID:
+            if constexpr (DG) return cudaErrorInvalidValue;
+            else return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_RESID, DG, LR>, a);
         case OP_PHI_REAL: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_PHI_REAL, DG, LR>, a);
         case OP_PHI_PAIR2: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_PHI_PAIR2, DG, LR>, a);
         case OP_P_REAL: return cudaLaunchKernelEx(&cfg, k_spmv_step<T, OP_P_REAL, DG, LR>, a);

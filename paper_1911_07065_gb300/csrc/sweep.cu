@@ -318,7 +318,7 @@ int32_t sweep_run_chain(const ppg_sweep_plan* P, const std::vector<Step>& plan,
         a.c1 = (float)st.c1;
         a.c2 = (float)st.c2;
         a.c3 = (float)st.c3;
-        a.flags = st.flags;
+        a.flags = st.flags | row_flags(n, P->nnz);
         const int32_t g = launch_step<float>(st.op, a, s);
         if (g < 0) return g;
     }
