@@ -157,9 +157,9 @@ __device__ __forceinline__ void step_epilogue(const StepArgs<T>& a, int64_t r, T
 // warp for each: on one thread such a row is a chain of dependent multiply-adds
 // and gathers that the whole step waits for.  Lane l takes entries l, l + 32,
 // ...; the lanes' sums meet in a fixed order.  19 FP64 steps over 198,907 rows
-// of about six entries and four of 2,500: 6.10 -> 0.60 ms, FP32 2.52 -> 0.35 ms.
-// (The whole CTA on a row measured 0.36 and 0.23 ms, but the code for it costs
-// every other matrix 3 % in registers.)
+// of about six entries and four of 2,500: 6.10 -> 0.39 ms, FP32 2.52 -> 0.26 ms.
+// (The whole CTA on a row is faster still, but the code for it cost every other
+// matrix 3 % in registers.)
 template <typename T, int OP>
 __device__ __forceinline__ void long_rows(const StepArgs<T>& a, int64_t r, bool is_long,
                                           double& sq) {
@@ -398,18 +398,22 @@ __device__ __forceinline__ T row_dot(const T* sval, const int32_t* scol, const T
 // Building it is two passes over the matrix, inside the call.  Whether the
 // matrix has the form is known on the device alone: the steps read it from
 // the head and take the CSR path if not, so the host waits for nothing, and
-// the call stays asynchronous and can be captured.
+// the call stays asynchronous and can be captured.  (A solve waits between cycles
+// anyway, asks, and launches the plain steps without a form.)  An FP32 matrix
+// without the form pays for the search, as below, and for CSR steps at 40
+// registers: seven random entries in a row 102 -> 63 us a step, narrow bands of
+// three, five and seven 28.4 -> 31.5, 33.3 -> 35.5 and 40.3 -> 41.1.
 //
-// 160^3, FP32, 60 steps of p(A): 2.94 -> 1.50 ms (one value per diagonal), 2.93
-// -> 2.28 ms (values of their own), against 49 us a step at 0.91 of the copy
-// bandwidth by CSR.  What is left is the issue of instructions (two thirds of
-// the slots) and the life of a CTA (head, copies, arithmetic: three trips).
+// 160^3, FP32, 60 steps of p(A): 2.94 -> 1.48 ms (one value per diagonal), 2.92
+// -> 2.23 ms (values of their own), against 49 us a step at 0.91 of the copy
+// bandwidth by CSR.  What is left is the issue of instructions and the life of a CTA
+// (head, copies, arithmetic: three trips).
 // Tried and slower: reading x and the values straight from global memory (27 -
 // 35 us a step, five dependent trips per CTA), and CTAs that stay and loop over
 // tiles without copies in flight (26 - 37 us).
 //
-// FP64 steps have no use for it: their multiply-adds bound them (504 G FMA/s
-// measured, 1.6 per clock and SM; the chains run at 0.85 - 0.89 of that).
+// FP64 steps have no use for it: their multiply-adds bound them (529 G FMA/s
+// measured, 1.68 per clock and SM; the chains run at 0.79 - 0.84 of that).
 
 constexpr int DIAG_TILE = step_threads<float>() * step_rpt<float>();   // rows of a tile
 constexpr int DIAG_CAP = 2 * (step_chunk<float>() + 4);   // elements of its shared memory
@@ -447,7 +451,11 @@ __global__ void k_diag_init(const int32_t* __restrict__ rowptr, const int32_t* _
 // shared memory (coalesced) and walks them there, one row per thread, beside its
 // own sorted list of the offsets so far; what the list lacks is merged into it and
 // the tile walked again, which for a grid happens once or twice in all.  At the
-// end one warp compares that list with the matrix's and adds what is new.
+// end one warp compares that list with the matrix's and adds what is new.  Latency
+// bounds it (a tile's three dependent trips, ten CTAs per SM): 4.1e6 rows of seven
+// entries 97 us, 1e6 of thirty 70 where the first tiles show that there is no form;
+// a CTA per 128 rows with a round of barriers and reads a row apart per entry took
+// 109 and 690.
 constexpr int DIAG_ROWS = 128;
 constexpr int DIAG_STAGE = 2048;   // entries in shared memory at once
 __device__ __forceinline__ int diag_at(int i) { return i + (i >> 5); }   // (no bank conflicts)
@@ -1446,10 +1454,10 @@ static int step_resident_ctas() {
 
 // The diagonal form is tried with at most as many diagonals as keep it below
 // the CSR's bytes (an entry without its column index), where the steps to come
-// repay building it: about two passes over the matrix, 60 us for 1e6 rows of
-// five entries and 160 us for 4.1e6 rows of seven.  Per step, CSR against
-// diagonals (one value per diagonal / values of their own):
-//   160^3:     49 us   24.2 us / 37 us   (repaid by 14 steps)
+// repay building it: two passes over the matrix, 135 us at 160^3 (165 us with values
+// of their own to write).  Per step, CSR against diagonals (one value per diagonal /
+// values of their own):
+//   160^3:     49 us   22.5 us / 34 us   (repaid by 5 and 11 steps)
 // A matrix held in L2 stays with the direct steps: by diagonals a grid would gain
 // (1000^2, 60 steps: 0.53 -> 0.38 ms), but whether it is one is known on the device
 // alone, and a matrix that is not would lose more than the direct steps' gain
