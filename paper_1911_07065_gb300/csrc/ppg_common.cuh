@@ -131,8 +131,7 @@ enum StepFlag : int {
                    // diagonal form built by the kernel before it
     F_WIDE = 32,   // more than 5.5 entries in the average row
     F_LONG = 64,   // ... more than LONG_AVG (spmv_root.cu)
-    F_LATE = 128,  // direct step: lets the next one in when the previous one is done
-    F_SPREAD = 256, // more than SPREAD_AVG entries in the average row
+    F_SPREAD = 128, // more than SPREAD_AVG entries in the average row
 };
 
 // An FP32 matrix by its diagonals (spmv_root.cu), built on the device inside

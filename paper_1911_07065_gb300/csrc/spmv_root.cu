@@ -1170,7 +1170,9 @@ constexpr int SPREAD_ROWS = 4;
 constexpr double SPREAD_AVG = 22.0;
 constexpr int LATE_MAX = 10;            // (launch_step)
 
-template <typename T, int OP, int PRE, int MINB, bool HINT>
+// LATE: lets the next step in when the previous one is done (launch_step); chosen
+// inside the kernel it cost 40 steps at 1000^2 0.2 %
+template <typename T, int OP, int PRE, int MINB, bool HINT, bool LATE>
 __global__ void __launch_bounds__(SPMV_ROWS, MINB)
 k_spmv_direct(const __grid_constant__ StepArgs<T> a) {
     __shared__ double sred[SPMV_ROWS / 32];
@@ -1183,8 +1185,7 @@ k_spmv_direct(const __grid_constant__ StepArgs<T> a) {
         r = (r >> 5) * SPREAD_ROWS + (tid & 31);
         live = (tid & 31) < SPREAD_ROWS && r < a.n;
     }
-    const bool late = a.flags & F_LATE;
-    if (!late) asm volatile("griddepcontrol.launch_dependents;");
+    if constexpr (!LATE) asm volatile("griddepcontrol.launch_dependents;");
     int32_t k0 = 0, k1 = 0;
     T pv[PRE];
     int32_t pc[PRE];
@@ -1207,7 +1208,7 @@ k_spmv_direct(const __grid_constant__ StepArgs<T> a) {
     const unsigned longs = HINT ? 0 : __ballot_sync(0xffffffffu, k1 - k0 > LONG_ROW);
     // the vectors written by the previous step are complete and visible
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (late) asm volatile("griddepcontrol.launch_dependents;");
+    if constexpr (LATE) asm volatile("griddepcontrol.launch_dependents;");
     double sq = 0.0;
     const bool is_long = k1 - k0 > LONG_ROW;
     if (live) {
@@ -1534,16 +1535,22 @@ int32_t DiagStore::settle(void* pinned) {
     return PPG_OK;
 }
 
+template <typename T, int OP, int PRE, int MINB, bool HINT>
+static cudaError_t launch_late(cudaLaunchConfig_t& cfg, const StepArgs<T>& a, bool late) {
+    return late ? cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP, PRE, MINB, HINT, true>, a)
+                : cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP, PRE, MINB, HINT, false>, a);
+}
+
 template <typename T, int PRE, int MINB, bool HINT>
-static cudaError_t launch_direct(cudaLaunchConfig_t& cfg, int op, const StepArgs<T>& a) {
+static cudaError_t launch_direct(cudaLaunchConfig_t& cfg, int op, const StepArgs<T>& a, bool late) {
     switch (op) {
-        case OP_SPMV: return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_SPMV, PRE, MINB, HINT>, a);
-        case OP_RESID: return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_RESID, PRE, MINB, HINT>, a);
-        case OP_PHI_REAL: return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_PHI_REAL, PRE, MINB, HINT>, a);
-        case OP_PHI_PAIR2: return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_PHI_PAIR2, PRE, MINB, HINT>, a);
-        case OP_P_REAL: return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_P_REAL, PRE, MINB, HINT>, a);
-        case OP_P_PAIR1: return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_P_PAIR1, PRE, MINB, HINT>, a);
-        case OP_P_PAIR2: return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_P_PAIR2, PRE, MINB, HINT>, a);
+        case OP_SPMV: return launch_late<T, OP_SPMV, PRE, MINB, HINT>(cfg, a, late);
+        case OP_RESID: return cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_RESID, PRE, MINB, HINT, false>, a);
+        case OP_PHI_REAL: return launch_late<T, OP_PHI_REAL, PRE, MINB, HINT>(cfg, a, late);
+        case OP_PHI_PAIR2: return launch_late<T, OP_PHI_PAIR2, PRE, MINB, HINT>(cfg, a, late);
+        case OP_P_REAL: return launch_late<T, OP_P_REAL, PRE, MINB, HINT>(cfg, a, late);
+        case OP_P_PAIR1: return launch_late<T, OP_P_PAIR1, PRE, MINB, HINT>(cfg, a, late);
+        case OP_P_PAIR2: return launch_late<T, OP_P_PAIR2, PRE, MINB, HINT>(cfg, a, late);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -1604,6 +1611,7 @@ int32_t launch_step(int op, const StepArgs<T>& a_in, cudaStream_t s) {
         // 54.88 ms against 256 rows; 64 rows 69.5 ms); the residual keeps 256:
         // one partial sum per 256 rows
         const int sms = a.sms = a.sms ? a.sms : device_sm_count();
+        bool late = false;
         if (op != OP_RESID) {
             const int rows_d = a_in.n <= sms * DIRECT_SMALL_ROWS ? DIRECT_SMALL_ROWS : DIRECT_L2_ROWS;
             cfg.blockDim = dim3(rows_d);
@@ -1622,7 +1630,7 @@ int32_t launch_step(int op, const StepArgs<T>& a_in, cudaStream_t s) {
             // for one chain of 300^2 and 400^2, but 259 and 317 for the four of them,
             // at 240^2 250 instead of 131.)  500^2 in FP32, 13 CTAs per SM, loses by
             // it: 116 -> 121 us.
-            if (cfg.gridDim.x <= (unsigned)(LATE_MAX * sms)) a.flags |= F_LATE;
+            late = cfg.gridDim.x <= (unsigned)(LATE_MAX * sms);
         }
         // matrix in L2: entries preloaded before the dependency wait.
         // Up to 5.5 in the average row, five: FP64 at 40 registers (1536 threads
@@ -1640,15 +1648,15 @@ int32_t launch_step(int op, const StepArgs<T>& a_in, cudaStream_t s) {
         // (45^3 201 -> 137 us, seven 146 us; 53^3 247 -> 168 us, seven 203 us).
         cudaError_t ed;
         if (small)
-            ed = launch_direct<T, 8, 0, false>(cfg, op, a);
+            ed = launch_direct<T, 8, 0, false>(cfg, op, a, late);
         else if ((a_in.flags & F_WIDE) && !F32 && a_in.n <= sms * 8 * DIRECT_L2_ROWS)
-            ed = launch_direct<T, 8, 4, true>(cfg, op, a);
+            ed = launch_direct<T, 8, 4, true>(cfg, op, a, late);
         else if (a_in.flags & F_WIDE)
-            ed = launch_direct<T, 7, 6, true>(cfg, op, a);
+            ed = launch_direct<T, 7, 6, true>(cfg, op, a, late);
         else if (!F32 && op == OP_SPMV)
-            ed = cudaLaunchKernelEx(&cfg, k_spmv_direct<T, OP_SPMV, 5, 8, true>, a);
+            ed = launch_late<T, OP_SPMV, 5, 8, true>(cfg, a, late);
         else
-            ed = launch_direct<T, 5, 6, true>(cfg, op, a);
+            ed = launch_direct<T, 5, 6, true>(cfg, op, a, late);
         ++g_launches;
         if (ed != cudaSuccess) {
             set_cuda_error(ed, "cudaLaunchKernelEx(k_spmv_direct)");
