@@ -285,17 +285,20 @@ bool cluster_possible() {
 
 // The line, from 40 steps of p(A), launch by launch / in one cluster.  FP64: where
 // the cluster's multiply-adds (nnz + n a step) take less than a step's launch: 2-D
-// 50^2 79 / 43 us, 80^2 78 / 65, 90^2 78 / 77, 100^2 77 / 83; 3-D 18^3 78 / 64, 20^3
-// 79 / 79.  As a graph the launches cost less: 70^2 64 / 57, 80^2 64 / 68.  FP32: up
-// to two rows a thread (50^2 76 / 22, as a graph 45 / 26; 128^2 78 / 37 and 47 /
-// 40).  And at most CHAIN_E entries in the average row: what a row has beyond them is
-// read again in each step, with the chain of its gathers in the cluster's few warps
-// (FP64, 2,000 rows of 30: 160 / 236 us, 220 rows of 200: 620 / 2,330; FP32, 3,000
-// rows of 64: 248 / 460).
+// 50^2 78 / 41 us, 85^2 79 / 68, 95^2 79 / 78, 98^2 78 / 83; short chains, where what a
+// call costs beside its launches counts, a little further (98^2, 20 steps of phi 45 /
+// 41).  As a graph the launches cost less: 70^2 64 / 57, 80^2 64 / 66.  FP32: up to two
+// rows a thread (50^2 76 / 21, as a graph 45 / 25; 128^2 78 / 35 and 47 / 39).  And at
+// most CHAIN_E entries in the average row: what a row has beyond them is read again
+// in each step, with the chain of its gathers in the cluster's few warps (FP64, 2,000
+// rows of 30: 160 / 236 us, 220 rows of 200: 620 / 2,330; FP32, 3,000 rows of 64: 248 /
+// 460).
 template <typename T>
 bool chain_cluster_fits(size_t steps, int32_t n, int64_t nnz, cudaStream_t s) {
     if (n > CHAIN_CTAS * CHAIN_THREADS * CHAIN_ROWS || nnz > (int64_t)CHAIN_E * n) return false;
-    if (sizeof(T) == 8 && nnz + n > 36000 && (nnz + n > 48000 || stream_capturing(s))) return false;
+    const int64_t work = nnz + n;
+    if (sizeof(T) == 8 && work > (steps <= 20 ? 60000 : 54000)) return false;
+    if (sizeof(T) == 8 && work > 36000 && stream_capturing(s)) return false;
     if (steps < 2 || steps > (size_t)CHAIN_STEPS) return false;
     return cluster_possible<T>();
 }
