@@ -82,7 +82,8 @@ def _ncu_traffic():
 
 def _inchain_ratio(profile, key):
     """DRAM bytes / algorithmic bytes of mid-chain root steps, from a
-    committed in-chain ncu summary (None if absent)."""
+    committed in-chain ncu summary (None if absent); any figure of a
+    summary that stands behind `key:`."""
     path = os.path.join(ROOT, "profiles", profile)
     if not os.path.exists(path):
         return None
@@ -390,6 +391,8 @@ def run_ours(args, rank, local, world):
     clk_mhz = clk.get("sm_mhz") or 2070.0
     fma_per_launch = P.A.nnz + P.A.n
     fp64_peak = 2.0 * sms * clk_mhz * 1e-3   # G FMA / s at the sampled SM clock
+    fp64_rate = _inchain_ratio("fp64_rate.md", "fp64_gfma_s_at_2070_mhz")   # what multiply-adds reach
+    fp64_rate = fp64_rate * clk_mhz / 2070.0 if fp64_rate else None
     fp64_achieved = poly_launches * fma_per_launch / (poly_ms * 1e-3) / 1e9 if poly_ms > 0 else None
     traffic = _ncu_traffic()
     ratio_c2 = _inchain_ratio("inchain_spmv_root_cd2d_1000.md", "dram_to_algorithmic_phi_f64")
@@ -457,6 +460,9 @@ def run_ours(args, rank, local, world):
                               "achieved_gfma_s": round(fp64_achieved, 1) if fp64_achieved else None,
                               "peak_gfma_s": round(fp64_peak, 1),
                               "frac": round(fp64_achieved / fp64_peak, 4) if fp64_achieved else None,
+                              "measured_gfma_s": round(fp64_rate, 1) if fp64_rate else None,
+                              "frac_of_measured": (round(fp64_achieved / fp64_rate, 4)
+                                                   if fp64_achieved and fp64_rate else None),
                               "peak_note": "2 FP64 FMA per clock per SM (ncu dfma peak) x %d SMs x "
                                            "the median SM clock sampled in the timed region" % sms}},
         "e2e": {"value": round(e2e, 3), "unit": UNIT, "h2d_bytes_per_step": int(h2d),
@@ -691,8 +697,8 @@ def measure_forms(device, with_oracle=True):
     As = P.A.to_scipy()
     xh32, xh64 = x32.cpu().numpy(), x64.cpu().numpy()
     out["precision_cd3d_160"] = {
-        "p_fp32_roofline": chain_bw(f32t, "p(A) v_j in FP32 (Algorithm 3), every outer step; "
-                                    "in bytes of the CSR, most of which the diagonal form does not read",
+        "p_fp32_roofline": chain_bw(f32t, "p(A) v_j in FP32 (Algorithm 3), every outer step; by "
+                                    "diagonals, in the bytes of that form (a mask and the vectors)",
                                     "dram_to_algorithmic_p_f32"),
         "phi_fp64_roofline": chain_bw(f64t, "phi(A) v_j in FP64 (Algorithm 1) and p(A) u per restart",
                                       "dram_to_algorithmic_phi_f64"),
