@@ -73,7 +73,7 @@ __device__ __forceinline__ void cluster_wait() {
 }
 
 template <typename T, int R>
-__global__ void __launch_bounds__(CHAIN_THREADS, 1)
+__global__ void __launch_bounds__(CHAIN_THREADS, R == 1 ? 1 : 0)
 k_chain_cluster(const __grid_constant__ ChainArgs<T> a) {
     extern __shared__ __align__(16) unsigned char chain_x[];   // 2 x chunk of T
     T* const xs = reinterpret_cast<T*>(chain_x);
@@ -146,20 +146,29 @@ k_chain_cluster(const __grid_constant__ ChainArgs<T> a) {
                 if (e < most) {   // uniform: no FP64 issue for what no lane has
                     if (e < ordinary) acc = fma(v[i][e], x[e], acc);
                 }
-            for (int e = CHAIN_E; e < ordinary; e += 4) {
-                // (past the end: the last entry again, so that the loads need no branch)
-                int32_t c[4];
-                T w[4], xe[4];
+            if constexpr (R == 1) {
+                for (int e = CHAIN_E; e < ordinary; e += 4) {
+                    // (past the end: the last entry again, so that the loads need no branch)
+                    int32_t c[4];
+                    T w[4], xe[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    c[u] = __ldg(a.colind + k0[i] + min(e + u, ordinary - 1));
-                    w[u] = __ldg(a.vals + k0[i] + min(e + u, ordinary - 1));
+                    for (int u = 0; u < 4; ++u) {
+                        c[u] = __ldg(a.colind + k0[i] + min(e + u, ordinary - 1));
+                        w[u] = __ldg(a.vals + k0[i] + min(e + u, ordinary - 1));
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) ld_cluster(xe[u], at(c[u]) + cur);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (e + u < ordinary) acc = fma(w[u], xe[u], acc);
                 }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) ld_cluster(xe[u], at(c[u]) + cur);
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (e + u < ordinary) acc = fma(w[u], xe[u], acc);
+            } else {   // (no registers for four at a time beside two rows)
+#pragma unroll 4
+                for (int e = CHAIN_E; e < ordinary; ++e) {
+                    T xe;
+                    ld_cluster(xe, at(__ldg(a.colind + k0[i] + e)) + cur);
+                    acc = fma(__ldg(a.vals + k0[i] + e), xe, acc);
+                }
             }
             // rows of more than LONG_ROW entries, a warp for each
             for (unsigned todo = longs[i]; todo; todo &= todo - 1) {

@@ -166,3 +166,31 @@ assert torch.equal(p.apply_poly(A, R, v), y)
 """
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     subprocess.run([sys.executable, "-c", code], check=True, cwd=root, timeout=300)
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("n", [300, 4000, 9000, 16384])
+def test_rows_beyond_the_registers_in_one_cluster(env, n, dtype):
+    """Rows of nine to some hundred entries among short ones, one and (above 8,192 rows,
+    FP32) two rows to a thread, against the same rows step by step."""
+    p, torch = env
+    tdt = torch.float64 if dtype == "f64" else torch.float32
+    if dtype == "f64" and n > 9000:
+        pytest.skip("more multiply-adds than the FP64 cluster takes")
+    lens = np.where(np.arange(n) % 97 == 5, 90, np.where(np.arange(n) % 31 == 7, 9 + np.arange(n) % 12, 3))
+    lens[[0, n - 1]] = 30, 140
+    rng = np.random.default_rng(3)
+    cols = [np.unique(np.concatenate([rng.integers(0, n, k - 1), [i]])) for i, k in enumerate(lens)]
+    rowptr = np.concatenate([[0], np.cumsum([c.size for c in cols])]).astype(np.int32)
+    H = synth.CSRHost(n, rowptr, np.concatenate(cols).astype(np.int32), 0.1 * rng.standard_normal(rowptr[-1]))
+    A = dev_csr(p, torch, H, dtype=tdt)
+    extra = 40000 - n
+    big = p.CSR(torch.cat([A.rowptr, A.nnz + torch.arange(1, extra + 1, dtype=torch.int32, device="cuda")]),
+                torch.cat([A.colind, A.n + torch.arange(extra, dtype=torch.int32, device="cuda")]),
+                torch.cat([A.vals, torch.full((extra,), 5.0, dtype=tdt, device="cuda")]))
+    assert p.chain_form(A, 33) == "cluster" and p.chain_form(big, 33) == "direct"
+    v = to_dev(torch, rng.standard_normal(n), tdt)
+    vb = torch.cat([v, torch.ones(extra, dtype=tdt, device="cuda")])
+    R = p.Roots.from_complex(_roots())
+    assert torch.equal(p.apply_poly(A, R, v), p.apply_poly(big, R, vb)[:n])
+    assert torch.equal(p.apply_phi(A, R, v), p.apply_phi(big, R, vb)[:n])
