@@ -1168,7 +1168,7 @@ constexpr int DIRECT_L2_ROWS = 128;     // ... above that
 // 10,000 of 18 89 / 110).
 constexpr int SPREAD_ROWS = 4;
 constexpr double SPREAD_AVG = 22.0;
-constexpr int LATE_MAX = 10;            // (launch_step)
+constexpr int LATE_MAX = 6, EVEN_MAX = 10;   // CTAs per SM (launch_step)
 
 // LATE: lets the next step in when the previous one is done (launch_step); chosen
 // inside the kernel it cost 40 steps at 1000^2 0.2 %
@@ -1619,18 +1619,25 @@ int32_t launch_step(int op, const StepArgs<T>& a_in, cudaStream_t s) {
             if (small && (a.flags & F_SPREAD))   // more warps for the same rows
                 threads = ((int64_t)a_in.n + SPREAD_ROWS - 1) / SPREAD_ROWS * 32;
             cfg.gridDim = dim3((unsigned)((threads + rows_d - 1) / rows_d));
-            // The next step is let in by a grid of at most LATE_MAX CTAs per SM only
-            // when the previous one is done, by a larger one at once.  At once, the
-            // CTAs of a third and fourth step come in too wherever there is room, to
-            // wait there, and a small step then starts with several CTAs on some SMs
-            // and none on others.  40 FP64 steps at once / so: 2-D 150^2 155 / 85 us,
-            // 240^2 217 / 103, 300^2 216 / 135, 400^2 223 / 163; four such chains on
-            // four streams, as graphs: 300^2 182 / 178 us, 400^2 316 / 315.  (Shared
-            // memory that leaves an SM room for its share only takes 104 and 147 us
-            // for one chain of 300^2 and 400^2, but 259 and 317 for the four of them,
-            // at 240^2 250 instead of 131.)  500^2 in FP32, 13 CTAs per SM, loses by
-            // it: 116 -> 121 us.
-            late = cfg.gridDim.x <= (unsigned)(LATE_MAX * sms);
+            // The next steps' CTAs take places wherever there is room before a step's own
+            // are done, to wait there, and a step of a few CTAs per SM then runs with
+            // several on some SMs and none on others.  So a grid of at most LATE_MAX
+            // CTAs per SM lets the next one in only when the previous one is done, so
+            // that at most one waits: 40 FP64 steps, let in at once / so, 2-D 150^2 155 /
+            // 85 us, 240^2 217 / 101, 300^2 216 / 135; four such chains on four streams, as
+            // graphs, 240^2 153 / 131, 300^2 182 / 178.  A larger one, up to EVEN_MAX, takes
+            // shared memory that nothing uses, which leaves an SM room for its share only:
+            // 350^2 211 us at once, 161 let in late, 131 so, the four 242, 241 and 273; 400^2
+            // 220, 163 and 148, the four 316, 315 and 317.  (Smaller grids gain by that too,
+            // 300^2 104 us, but shut other streams out: the four 260 us, at 240^2 251.)
+            // Above, neither pays (500^2 in FP32, 13 CTAs per SM, let in late 116 -> 121 us).
+            const int per = (int)((cfg.gridDim.x + sms - 1) / sms);
+            late = per <= LATE_MAX;
+            // 228 KB per SM, 1 KB of it taken by each CTA beside its own; a share and
+            // one CTA more must not fit (eight of 64 registers a thread do not)
+            const bool by_registers = (a_in.flags & F_WIDE) && !F32 && a_in.n <= sms * 8 * DIRECT_L2_ROWS;
+            if (!small && !late && per <= EVEN_MAX && !by_registers)
+                cfg.dynamicSmemBytes = (size_t)(228 / per - 2) * 1024;
         }
         // matrix in L2: entries preloaded before the dependency wait.
         // Up to 5.5 in the average row, five: FP64 at 40 registers (1536 threads
